@@ -64,7 +64,10 @@ typedef struct {
 
 /* Resident-DB layouts, chosen once at setup (the GEMM path follows the layout). */
 typedef enum {
-  PIR_LAYOUT_PLAIN = 0,  /* u32 residues [L*n slots][D1][D2]: CUDA-core u32 x u32 -> u64 path */
+  PIR_LAYOUT_PLAIN = 0,  /* u32 residues [L*n slots][D1][D2]: one query on the CUDA cores (u32 x u32 ->
+                            u64), batches on the tensor cores (the words split into exact signed
+                            base-256 f16 digits on the way, 1024-row f32 sums of at most 2^24);
+                            tiles 1-8 keep a batch on the CUDA cores */
   PIR_LAYOUT_LIMB = 1,   /* u8 limb planes [L*n slots][4][D2][D1]: INT8 tensor-pipe path    */
   PIR_LAYOUT_TENSOR = 2  /* signed base-256 digits in bf16, 8 bytes per residue, laid out as
                             tensor-core operand tiles: the tcgen05 bf16 path (needs
@@ -129,7 +132,9 @@ typedef struct {
                         this many ciphertexts (bounds the scratch to one chunk)     */
   uint32_t tile;     /* 0 = built-in choice; else a GEMM tile id (pir_gemm_tiles) that
                         holds the batch: plain 1, 2, 3 and 7 take at most 2, 4, 8 and
-                        8 query rows (2B), 7 also D2 <= 512; limb 2 and 3 need the
+                        8 query rows (2B), 7 also D2 <= 512, 9 (the tensor-core GEMM,
+                        the built-in choice for K-chunks of 128 rows and more) at
+                        least 3; limb 2 and 3 need the
                         rows padded to 16 to be multiples of 32 and 64; tensor 1 is
                         the 1-SM GEMM, 2 the CTA-pair (2-SM) GEMM, which needs
                         D2 % 64 == 0, 3 and 4 the 1-SM GEMM in clusters of 2 and 4

@@ -96,6 +96,7 @@ struct pir_session {
   void *mem;        // qhat | qs | out
   void *stage_mem;  // two host-piece staging buffers, allocated with the first host piece
   size_t qhat_bytes, qs_bytes, stage_bytes;
+  uint32_t digit_rows;  // the digit GEMM's pieces, or 0
   cudaEvent_t arrived[2], consumed[2];
 };
 
@@ -211,6 +212,21 @@ uint32_t layout_chunk(int layout, uint32_t Kc) {
 // four bf16 digits
 size_t layout_qs_bytes(int layout, uint64_t nslots, uint32_t Kc, uint32_t Mp) {
   return (size_t)nslots * Kc * Mp * (layout == PIR_LAYOUT_TENSOR ? 8 : 4);
+}
+// The query copy of chunks of Kc rows under a tile choice: its bytes, and for the plain
+// layout's digit GEMM the rows of the pieces it takes a chunk in (else 0).  tight: within
+// the bytes that the other tiles take.
+struct QueryCopy {
+  size_t bytes;
+  uint32_t rows;
+};
+QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t Mp, uint32_t D2,
+                     bool tight) {
+  const size_t b = layout_qs_bytes(layout, nslots, Kc, Mp);
+  if (layout != PIR_LAYOUT_PLAIN || !gemm_plain_uses_digits(tile, M, Kc, D2)) return {b, 0};
+  const uint32_t rows = gemm_digit_rows(nslots, Kc, Mp, tight);
+  const size_t d = gemm_digit_query_bytes(nslots, rows, Mp);
+  return {d > b ? d : b, rows};
 }
 uint32_t layout_tiles(int layout) {
   return layout == PIR_LAYOUT_PLAIN ? gemm_plain_tiles() : layout == PIR_LAYOUT_LIMB ? gemm_limb_tiles()
@@ -328,10 +344,26 @@ struct StageTimer {
 
 // One K-chunk on the DB's GEMM path: the NTT-form chunk qhat [B][kc][2][L][n] to
 // the layout's query copy qs, then the GEMM accumulated into out [L*n][M][D2].
+// digit_rows: the plain layout's digit GEMM in pieces of so many rows (query_copy).
 pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint32_t Mp, uint32_t i0, uint32_t kc,
-                        void *qs, uint32_t *out, uint32_t tile, int stall, StageTimer &tm, cudaStream_t s) {
+                        uint32_t digit_rows, void *qs, uint32_t *out, uint32_t tile, int stall, StageTimer &tm,
+                        cudaStream_t s) {
   const ParamCtx &c = *db->ctx;
   const uint32_t D1 = db->p.D1, D2 = db->p.D2, M = 2 * B;
+  if (digit_rows) {
+    uint16_t *qt = static_cast<uint16_t *>(qs);
+    for (uint32_t k0 = 0; k0 < kc; k0 += digit_rows) {
+      const uint32_t kr = kc - k0 < digit_rows ? kc - k0 : digit_rows;
+      tm.begin();
+      CK(launch_query_digits(c, qhat, B, kc, k0, kr, Mp, qt, s));
+      tm.end(1, 1);
+      tm.begin();
+      CK(launch_gemm_digit(c, static_cast<const uint32_t *>(db->resident), D1, D2, qt, M, Mp, i0 + k0, kr, out,
+                           i0 + k0 > 0, s));
+      tm.end(2, 1);
+    }
+    return PIR_OK;
+  }
   tm.begin();
   if (db->layout == PIR_LAYOUT_PLAIN)
     CK(launch_query_to_slots(c, qhat, B, kc, Mp, static_cast<uint32_t *>(qs), s));
@@ -422,7 +454,9 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
 
   // scratch: NTT'd query chunk | slot-major query chunk | slot-major results
   const size_t qhat_bytes = qhat_ready ? 0 : (size_t)B * Kc * 2 * L * n * 4;
-  const size_t qs_bytes = layout_qs_bytes(db->layout, nslots, Kc, Mp);
+  // (the stall test hook belongs to the TMA scan)
+  const uint32_t qtile = stall ? 7 : o.tile;
+  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, Mp, D2, false);
   const size_t out_bytes = nslots * M * D2 * 4;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   // Batch 1 on the TMA scan: the forward NTT writes the slot layout itself (pairs of
@@ -438,7 +472,15 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   // K-chunked fused path: the chunks before the last accumulate slot-major here
   const size_t slot_bytes = (fused && Kc < D1) ? out_bytes : 0;
   Scratch scratch(s);
-  CK(scratch.alloc(up(qhat_bytes) + up(qs_bytes) + up(out_bytes) + up(full_bytes) + up(slot_bytes)));
+  const size_t other_bytes = up(qhat_bytes) + up(out_bytes) + up(full_bytes) + up(slot_bytes);
+  cudaError_t ae = scratch.alloc(other_bytes + up(qc.bytes));
+  if (ae == cudaErrorMemoryAllocation && qc.rows) {
+    cudaGetLastError();
+    qc = query_copy(db->layout, qtile, nslots, Kc, M, Mp, D2, true);
+    ae = scratch.alloc(other_bytes + up(qc.bytes));
+  }
+  CK(ae);
+  const size_t qs_bytes = qc.bytes;
   char *base = static_cast<char *>(scratch.ptr);
   const uint32_t *qhat = qhat_ready ? qhat_ready : reinterpret_cast<uint32_t *>(base);
   void *qs = base + up(qhat_bytes);
@@ -500,7 +542,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
                              s));
       tm.end(0, 1);
     }
-    const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, qs, out, o.tile, stall, tm, s);
+    const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, qc.rows, qs, out, o.tile, stall, tm, s);
     if (st != PIR_OK) return st;
   }
   tm.begin();
@@ -571,7 +613,7 @@ pir_status_t session_piece(pir_session *ses, const uint32_t *src, uint64_t strid
   CK(launch_ntt_fwd_rows(c, src, 0, G, row_stride, qhat, (uint64_t)B * G, s));
   tm.end(0, 1);
   if (!on_device) CK(cudaEventRecord(ses->consumed[slot], s));
-  const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, qs, out, ses->o.tile, 0, tm, s);
+  const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, ses->digit_rows, qs, out, ses->o.tile, 0, tm, s);
   if (st != PIR_OK) return st;
   if (!on_device) CK(cudaEventSynchronize(ses->arrived[slot]));  // the caller's buffer is free again
   return PIR_OK;
@@ -644,11 +686,18 @@ pir_status_t session_open(pir_db *db, uint32_t B, uint32_t kc_max, cudaStream_t 
   ses->o = o;
   ses->failed = PIR_OK;
   ses->qhat_bytes = (size_t)B * kc_max * ct * 4;
-  ses->qs_bytes = layout_qs_bytes(db->layout, nslots, kc_max, Mp);
+  QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, Mp, p.D2, false);
   ses->stage_bytes = up(ses->qhat_bytes);
   const size_t out_bytes = nslots * M * p.D2 * 4;
   void *mem = nullptr;
-  cudaError_t e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(ses->qs_bytes) + up(out_bytes), s);
+  cudaError_t e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
+  if (e == cudaErrorMemoryAllocation && qc.rows) {
+    cudaGetLastError();
+    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, Mp, p.D2, true);
+    e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
+  }
+  ses->qs_bytes = qc.bytes;
+  ses->digit_rows = qc.rows;
   if (e == cudaSuccess) ses->mem = mem;
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
     if ((e = cudaEventCreateWithFlags(&ses->arrived[k], cudaEventDisableTiming)) == cudaSuccess)
@@ -1410,6 +1459,7 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
     if (M <= 2) tiles.push_back(1);
     if (M <= 4) tiles.push_back(2);
     if (M <= 8) tiles.push_back(3);
+    if (gemm_plain_tile_ok(kDigitTile, M, p.D2)) tiles.push_back(kDigitTile);
     for (uint32_t t = 4; t <= 6; ++t) tiles.push_back(t);
     if (scan_tma_supports(M, p.D2)) tiles.push_back(7);
   } else {

@@ -302,13 +302,16 @@ cudaError_t gemm_launch(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint
 
 // Tile ids: 1 = GEMV MB=2, 2 = GEMV MB=4, 3 = GEMV MB=8, 4 = GEMM 16x256, 5 = GEMM 32x256,
 // 6 = GEMM 64x128, 7 = TMA-staged scan (M <= 8, D2 <= 512; scan_tma.cu), 8 = GEMM 8x256
-// (one query row per thread, for a few queries).  0 picks the TMA scan up to 4 rows,
-// the 8-row GEMM up to 8, else a GEMM tile by M.
-uint32_t gemm_plain_tiles() { return 8; }
+// (one query row per thread, for a few queries).  Where the digit GEMM does not apply, 0
+// picks the TMA scan up to 4 rows, the 8-row GEMM up to 8, else a GEMM tile by M.
+// 9 = the tensor-core GEMM over in-kernel digits (gemm_digit.cu), which takes another
+// query operand and is launched by its own entry point.
+uint32_t gemm_plain_tiles() { return kDigitTile; }
 
 bool gemm_plain_tile_ok(uint32_t tile, uint32_t M, uint32_t D2) {
   switch (tile) {
     case 0: case 4: case 5: case 6: case 8: return true;
+    case kDigitTile: return M >= 3 && gemm_digit_available();  // one query streams the DB at HBM speed already
     case 1: return M <= 2;
     case 2: return M <= 4;
     case 3: return M <= 8;

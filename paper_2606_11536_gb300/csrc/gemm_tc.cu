@@ -47,6 +47,7 @@
 
 #include "async.cuh"
 #include "common.cuh"
+#include "tcgen.cuh"
 
 namespace gbpir {
 namespace {
@@ -874,7 +875,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// A digit array [blocks][groups][128] (bf16 bits; a group = 8 rows x 16 K values, one
+bool tensor_maps_available() { return tensor_map_encoder() != nullptr; }
+
+// A digit array [blocks][groups][128] (16-bit elements; a group = 8 rows x 16 K values, one
 // core-matrix pair) as a 3-D tensor map with boxes of box_groups groups x box_blocks
 // blocks.  False if the encoder refuses it (or is missing).
 bool digit_tensor_map(CUtensorMap *map, const uint16_t *base, uint64_t groups, uint64_t blocks, uint32_t box_groups,
@@ -887,6 +890,19 @@ bool digit_tensor_map(CUtensorMap *map, const uint16_t *base, uint64_t groups, u
   const cuuint32_t estride[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<uint16_t *>(base), dims, strides, box, estride,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool word_tensor_map(CUtensorMap *map, const uint32_t *base, uint64_t cols, uint64_t rows, uint64_t slots,
+                     uint32_t box_rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return false;
+  const cuuint64_t dims[3] = {cols, rows, slots};
+  const cuuint64_t strides[2] = {cols * 4, cols * rows * 4};
+  const cuuint32_t box[3] = {32, box_rows, 1};
+  const cuuint32_t estride[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t *>(base), dims, strides, box, estride,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
