@@ -370,18 +370,19 @@ pir_status_t pir_fold(const pir_params_t *params, const uint32_t *cts, uint32_t 
 pir_status_t pir_answer_folded(pir_db_t db, const uint32_t *queries, uint32_t B, uint32_t ell, const uint32_t *rgsw,
                                uint32_t *responses, int on_device, void *stream, const pir_answer_opts_t *opts);
 
-/* Scalar-HE (LWE) DB GEMM of SimplePIR's online step (Sec. 2.5), built as Sec. 4.1
- * builds it on the INT8 tensor pipe:
+/* Scalar-HE (LWE) DB GEMM of SimplePIR's online step (Sec. 2.5), decomposed as in Sec. 4.1:
  *     out[b][i] = sum_j db[i][j] * queries[b][j]   (mod 2^32)
  *   db:      [D1][D0] int8 (signed plaintexts; the raw DB, no encoding), device.
  *   queries: [B][D0] uint32 (the query ciphertexts' Z_2^32 entries), device.
  *   out:     [B][D1] uint32, device, written.
- * Each query word is split into four byte planes (prmt), each plane multiplied on
- * the tensor pipe (mma.sync s8 x u8 -> s32, wrapping = mod 2^32) and the planes
- * recombined by shifts.  path: PIR_LWE_TENSOR, PIR_LWE_SIMT (CUDA-core dp4a on the
- * same byte planes), or PIR_LWE_AUTO (tensor from 8 queries up).  D0 must be a
- * multiple of 16 and at most 2^24; buffers 16-byte aligned.  Asynchronous on
- * stream; the caller owns every buffer.
+ * Each query word is split into four base-256 digits, each digit multiplied with the DB
+ * and the sums recombined by shifts (wrapping = mod 2^32).  path: PIR_LWE_TENSOR
+ * (tcgen05 f16, signed digits, exact 1024-byte f32 sums; the query digits take scratch
+ * from the stream-ordered allocator, 8 bytes per query word, without which the
+ * CUDA-core path answers), PIR_LWE_SIMT (CUDA-core dp4a on byte planes), or
+ * PIR_LWE_AUTO (the faster of the two for these sizes).  D0 must be a multiple of 16
+ * and at most 2^24; buffers 16-byte aligned.  Asynchronous on stream; the caller owns
+ * every buffer.
  * Errors: PIR_ERR_ARG (NULL or misaligned buffers, zero or unsupported sizes, unknown
  * path), PIR_ERR_CUDA. */
 #define PIR_LWE_AUTO 0u

@@ -67,6 +67,20 @@ pir_status_t cuda_status(cudaError_t e) {
   return PIR_ERR_CUDA;
 }
 
+// Keep the pool's memory once freed: repeated answers then reuse it instead of
+// returning it to the driver every call (pir_release_memory gives it back).
+void keep_pool_memory(int dev) {
+  static std::once_flag once[64];
+  if (dev < 0 || dev >= 64) return;
+  std::call_once(once[dev], [dev]() {
+    cudaMemPool_t pool;
+    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+      uint64_t thr = ~0ull;
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    }
+  });
+}
+
 }  // namespace gbpir
 
 using namespace gbpir;
@@ -236,19 +250,6 @@ bool layout_tile_ok(int layout, uint32_t tile, uint32_t M, uint32_t Mp, uint32_t
   if (layout == PIR_LAYOUT_PLAIN) return gemm_plain_tile_ok(tile, M, D2);
   if (layout == PIR_LAYOUT_LIMB) return gemm_limb_tile_ok(tile, Mp);
   return gemm_tc_tile_ok(tile, Mp, D2);
-}
-
-// Keep the pool's memory once freed: repeated answers then reuse it instead of
-// returning it to the driver every call.
-void keep_pool_memory(int dev) {
-  static std::once_flag once;
-  std::call_once(once, [dev]() {
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-      uint64_t thr = ~0ull;
-      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-    }
-  });
 }
 
 // Device memory an allocation can draw on: free memory plus what the stream-ordered

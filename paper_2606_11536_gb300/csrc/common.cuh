@@ -105,6 +105,7 @@ struct DbView {
 };
 bool db_view(pir_db_t db, DbView *out);
 void count_launches(uint64_t k);
+void keep_pool_memory(int dev);
 
 // Error bookkeeping (api.cu)
 // Per-device error word that kernels with bounded waits set on a timeout.
@@ -162,6 +163,11 @@ cudaError_t launch_gemm_plain(const ParamCtx &c, const uint32_t *db, uint32_t D1
                               uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
                               uint32_t tile, int stall_test, cudaStream_t s);
 uint32_t gemm_plain_tiles();
+
+// lwe_tc.cu: the scalar-HE product on the tensor cores; qt is scratch for the query digits.
+size_t lwe_tc_scratch_bytes(uint32_t D0, uint32_t B);
+cudaError_t launch_lwe_tc(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
+                          uint16_t *qt, cudaStream_t s);
 
 // gemm_digit.cu: the same contract on the tensor cores, the DB words split into digits
 // on the way (tile 9 of the plain layout).  Its query operand is f16 digits

@@ -69,10 +69,9 @@ constexpr uint32_t kRows = 64;                    // DB rows per block
 constexpr uint32_t kRawBytes = kRows * 32 * 4;    // one block of DB words
 constexpr uint32_t kBlockCols = kRows / 2;        // tensor-memory columns of one block's digits
 constexpr uint32_t kChunkRows = 1024;             // rows per exact f32 sum
-constexpr uint32_t kMaxRaw = 16, kMaxB = 4, kMaxA = 8;
+constexpr uint32_t kMaxRaw = 16, kMaxB = 4, kMaxA = 4;
 constexpr uint32_t kTmem = 512;
 constexpr uint32_t kBars = 2 * kMaxRaw + 2 * kMaxB + 2 * kMaxA + 2 * 3 + 1;
-constexpr uint32_t kSmemMax = 227u << 10, kSmemMin = 116u << 10;  // above half an SM: one CTA per SM
 
 struct DigArgs {
   uint32_t *out;  // [L*n][M][D2]
@@ -106,18 +105,6 @@ __device__ __forceinline__ uint32_t ld_shared(uint32_t addr) {
   return v;
 }
 
-// A ring position: slot and the parity of its current round.
-struct Ring {
-  uint32_t slot = 0, phase = 0;
-  __device__ __forceinline__ void next(uint32_t size) {
-    if (++slot == size) slot = 0, phase ^= 1;
-  }
-  __device__ __forceinline__ void skip(uint32_t count, uint32_t size) {
-    slot += count;
-    while (slot >= size) slot -= size, phase ^= 1;
-  }
-};
-
 // The units first, first + step, ... of a CTA (or pair), divided out once.
 struct UnitWalk {
   uint32_t cg, mt, s, dcg, dmt, ds;
@@ -131,11 +118,6 @@ struct UnitWalk {
     if (mt >= a.mtiles) mt -= a.mtiles, ++s;
   }
 };
-
-__device__ __forceinline__ uint32_t half2_sub(uint32_t bits, uint32_t bias) {
-  const __half2 f = __hsub2(*reinterpret_cast<const __half2 *>(&bits), *reinterpret_cast<const __half2 *>(&bias));
-  return *reinterpret_cast<const uint32_t *>(&f);
-}
 
 template <int CG, int SUB>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -591,36 +573,6 @@ __global__ void __launch_bounds__(256) k_query_digits(const uint32_t *__restrict
 uint32_t round16(uint32_t x) { return (x + 15u) & ~15u; }
 uint32_t round64(uint32_t x) { return (x + 63u) & ~63u; }
 
-template <int CG, int SUB>
-cudaError_t digit_launch(const DigArgs &a, const ModConst &mod, const CUtensorMap &tm_db, const CUtensorMap &tm_q,
-                         size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_digit<CG, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CG;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(sms / CG * CG), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = CG == 2 ? 1 : 0;
-  int resident = sms / CG;
-  if (CG == 2 && (cudaOccupancyMaxActiveClusters(&resident, k_gemm_digit<CG, SUB>, &cfg) != cudaSuccess || resident <= 0)) {
-    cudaGetLastError();  // clear the query's error: one cluster per SM pair
-    resident = sms / CG;
-  }
-  if ((uint32_t)resident > a.nunits) resident = (int)a.nunits;
-  cfg.gridDim = dim3((unsigned)(resident * CG), 1, 1);
-  return cudaLaunchKernelEx(&cfg, k_gemm_digit<CG, SUB>, a, mod, tm_db, tm_q);
-}
-
 }  // namespace
 
 // Whole chunks while their digits stay within 1 GiB; longer ones in pieces whose digits
@@ -695,15 +647,16 @@ cudaError_t launch_gemm_digit(const ParamCtx &c, const uint32_t *db, uint32_t D1
   a.SB = kMaxB;
   while (a.SB > 2 && a.SB * a.bstage > 100u << 10) --a.SB;
   a.SR = (uint32_t)((kSmemMax - fixed - a.SB * a.bstage) / kRawBytes);
-  if (a.SR > kMaxRaw) a.SR = kMaxRaw;
+  a.SR = a.SR >= kMaxRaw ? kMaxRaw : 8;  // whole rounds of the converter groups: a slot stays with one group
   size_t smem = a.SR * kRawBytes + a.SB * a.bstage + fixed;
   if (smem < kSmemMin) smem = kSmemMin;
   alignas(64) CUtensorMap tm_db = {}, tm_q = {};
   if (!word_tensor_map(&tm_db, db, D2, D1, nslots, kRows) ||
       !digit_tensor_map(&tm_q, qt, Ntot / 8, nslots * a.Uc, a.NH / CG / 8, SUB * kRows / 16))
     return cudaErrorInvalidValue;
-  if (H == 2) return digit_launch<2, 1>(a, c.mod, tm_db, tm_q, smem, s);
-  return CG == 2 ? digit_launch<2, 2>(a, c.mod, tm_db, tm_q, smem, s) : digit_launch<1, 2>(a, c.mod, tm_db, tm_q, smem, s);
+  if (H == 2) return launch_persistent<k_gemm_digit<2, 1>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
+  return CG == 2 ? launch_persistent<k_gemm_digit<2, 2>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q)
+                 : launch_persistent<k_gemm_digit<1, 2>, 1>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
 }
 
 }  // namespace gbpir

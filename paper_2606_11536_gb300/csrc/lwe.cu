@@ -1,24 +1,16 @@
-// lwe.cu -- the scalar-HE (LWE) DB GEMM of SimplePIR's online step (Sec. 2.5) on the
-// INT8 tensor pipe, as Sec. 4.1 builds it:
+// lwe.cu -- the scalar-HE (LWE) DB GEMM of SimplePIR's online step (Sec. 2.5) on the CUDA
+// cores, and the choice between it and the tensor-core path (lwe_tc.cu):
 //     out[b][i] = sum_j A[i][j] * Q[b][j]   (mod 2^32)
 // with A the raw DB (D1 x D0 signed INT8 plaintexts, no NTT encoding, no bloating)
-// and Q the B query vectors of Z_{2^32} entries.  Every query word splits into four
-// byte planes Q_p (Q = sum_p 2^(8p) Q_p); each A Q_p is an s8 x u8 product with s32
-// accumulation, and out = sum_p (A Q_p) << 8p.  Wrapping 32-bit arithmetic is exactly
-// arithmetic mod 2^32, so the accumulators need no K chunking.
+// and Q the B query vectors of Z_{2^32} entries.  As Sec. 4.1 decomposes it, every query
+// word splits into four byte planes Q_p (Q = sum_p 2^(8p) Q_p); each A Q_p is an s8 x u8
+// product with s32 accumulation, and out = sum_p (A Q_p) << 8p.  Wrapping 32-bit
+// arithmetic is exactly arithmetic mod 2^32, so the accumulators need no K chunking.
 //
-// Tensor path: mma.sync m16n8k32 s8.u8 -> s32 (this toolkit has no tcgen05 INT8 for
-// sm_103a).  A warp owns 64 rows x 8 queries; its four n8 tiles are the four byte
-// planes of the same 8 queries, so one thread holds all planes of its outputs and
-// combines them with shifts.  The byte planes come straight from the staged query
-// words: for 4 consecutive words of one query, eight prmt (a 4 x 4 byte transpose)
-// give the four plane registers the B fragment wants.  A and Q tiles are staged by
-// cp.async into double-buffered shared memory (A swizzled for ldmatrix).
-//
-// CUDA-core path (small batches, where the n8 query tile would be mostly padding):
-// dp4a s8 x u8 over the same byte planes, one DB row per thread, the query planes
-// transposed once per stage in shared memory and read as broadcasts.
+// The products are dp4a: one DB row per thread, the query planes transposed once per
+// stage in shared memory (eight prmt per 4 x 4 bytes) and read as broadcasts.
 #include "common.cuh"
+#include "tcgen.cuh"
 
 namespace gbpir {
 namespace {
@@ -51,111 +43,6 @@ __device__ __forceinline__ void byte_planes(uint32_t w0, uint32_t w1, uint32_t w
 // A tile: rows of KS bytes, 16-byte chunks XOR-swizzled by row (ldmatrix without
 // bank conflicts).
 __device__ __forceinline__ uint32_t swz_a(uint32_t r, uint32_t ch) { return r * KS + ((ch ^ (r & 7)) << 4); }
-// Q tile: rows of KS words (512 B); chunk c of query n at c ^ (4 (n & 1)), so the
-// fragment reads of a quarter warp (two queries x four chunks) hit distinct banks.
-__device__ __forceinline__ uint32_t swz_q(uint32_t n, uint32_t c) { return n * KS * 4 + ((c ^ ((n & 1) << 2)) << 4); }
-
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-
-__device__ __forceinline__ void mma_s8u8(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k32.row.col.s32.s8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// CTA = 4 warps: WR along rows x WQ along queries; warp tile 64 rows x 8 queries.
-template <int WQ>
-__global__ void __launch_bounds__(128) k_lwe_mma(const int8_t *__restrict__ A, uint32_t D1, uint32_t D0,
-                                                 const uint32_t *__restrict__ Q, uint32_t B, uint32_t *__restrict__ out) {
-  constexpr int WR = 4 / WQ, TM = 64 * WR, TQ = 8 * WQ;
-  constexpr int A_BYTES = TM * KS, Q_BYTES = TQ * KS * 4, STAGE = A_BYTES + Q_BYTES;
-  extern __shared__ __align__(128) uint8_t smem[];
-  const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t wr = warp % WR, wq = warp / WR;
-  const uint64_t m0 = (uint64_t)blockIdx.x * TM;
-  const uint32_t q0 = blockIdx.y * TQ;
-
-  auto load_stage = [&](int buf, uint32_t k0) {
-    const uint32_t sbase = smem_addr(smem + buf * STAGE);
-    for (uint32_t t = tid; t < TM * (KS / 16); t += 128) {  // A: TM rows x 8 chunks
-      const uint32_t ch = t & 7, r = t >> 3;
-      const bool ok = (m0 + r < D1) && (k0 + ch * 16 < D0);
-      const int8_t *g = A + (m0 + r) * D0 + k0 + ch * 16;
-      cp16z(sbase + swz_a(r, ch), ok ? g : A, ok);
-    }
-    for (uint32_t t = tid; t < TQ * (KS / 4); t += 128) {  // Q: TQ queries x 32 chunks of 4 words
-      const uint32_t c = t & 31, n = t >> 5;
-      const bool ok = (q0 + n < B) && (k0 + c * 4 < D0);
-      const uint32_t *g = Q + (uint64_t)(q0 + n) * D0 + k0 + c * 4;
-      cp16z(sbase + A_BYTES + swz_q(n, c), ok ? g : Q, ok);
-    }
-    asm volatile("cp.async.commit_group;\n" ::);
-  };
-
-  int acc[4][4][4];  // [m16 tile][byte plane][fragment]
-#pragma unroll
-  for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) acc[mt][p][f] = 0;
-
-  const uint32_t nk = (D0 + KS - 1) / KS;
-  const uint32_t n_loc = wq * 8 + (lane >> 2), tg = lane & 3;
-  load_stage(0, 0);
-  for (uint32_t kt = 0; kt < nk; ++kt) {
-    const int buf = kt & 1;
-    asm volatile("cp.async.wait_group 0;\n" ::);
-    __syncthreads();
-    if (kt + 1 < nk) load_stage(buf ^ 1, (kt + 1) * KS);
-    const uint32_t sA = smem_addr(smem + buf * STAGE), sQ = sA + A_BYTES;
-#pragma unroll
-    for (int kk = 0; kk < KS / 32; ++kk) {
-      // B fragments of the four byte planes: words k = 32 kk + 4 tg + (0..3) and +16
-      uint32_t b0[4], b1[4];
-      {
-        uint4 lo, hi;
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n"
-                     : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w)
-                     : "r"(sQ + swz_q(n_loc, kk * 8 + tg)));
-        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n"
-                     : "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
-                     : "r"(sQ + swz_q(n_loc, kk * 8 + 4 + tg)));
-        byte_planes(lo.x, lo.y, lo.z, lo.w, b0);
-        byte_planes(hi.x, hi.y, hi.z, hi.w, b1);
-      }
-#pragma unroll
-      for (int mt = 0; mt < 4; ++mt) {
-        uint32_t a[4];
-        const uint32_t ar = wr * 64 + mt * 16 + (lane & 15), ach = 2 * kk + (lane >> 4);
-        ldsm_x4(sA + swz_a(ar, ach), a);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) mma_s8u8(acc[mt][p], a, b0[p], b1[p]);
-      }
-    }
-  }
-
-  // epilogue: out = sum_p acc_p << 8p (mod 2^32); fragment f: row g + 8 (f >> 1), query 2 tg + (f & 1)
-  const uint32_t g = lane >> 2;
-#pragma unroll
-  for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const uint64_t i = m0 + wr * 64 + mt * 16 + g + 8 * (f >> 1);
-      const uint32_t b = q0 + wq * 8 + 2 * tg + (f & 1);
-      if (i >= D1 || b >= B) continue;
-      uint32_t v = 0;
-#pragma unroll
-      for (int p = 0; p < 4; ++p) v += (uint32_t)acc[mt][p][f] << (8 * p);
-      out[(uint64_t)b * D1 + i] = v;
-    }
-}
-
 // CUDA-core path: 256 rows per CTA (one per thread) x QB queries.  Per stage the raw
 // query words are staged, then transposed once into planes [QB][KS/4][4] that every
 // thread reads as broadcasts.  blockIdx.z takes K stages [z * kper, (z + 1) * kper):
@@ -242,19 +129,6 @@ __global__ void __launch_bounds__(256) k_lwe_dp4a(const int8_t *__restrict__ A, 
   }
 }
 
-template <int WQ>
-cudaError_t mma_launch(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
-                       cudaStream_t s) {
-  constexpr int TM = 64 * (4 / WQ), TQ = 8 * WQ;
-  constexpr int smem = 2 * (TM * KS + TQ * KS * 4);
-  cudaError_t e = cudaFuncSetAttribute(k_lwe_mma<WQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const uint64_t gx = (D1 + TM - 1) / TM, gy = (B + TQ - 1) / TQ;
-  if (gx > 0x7FFFFFFFull || gy > 65535) return cudaErrorInvalidConfiguration;
-  k_lwe_mma<WQ><<<dim3((unsigned)gx, (unsigned)gy), 128, smem, s>>>(A, D1, D0, Q, B, out);
-  return cudaGetLastError();
-}
-
 template <int QB>
 cudaError_t dp4a_launch(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
                         cudaStream_t s, uint32_t *launches) {
@@ -287,19 +161,43 @@ cudaError_t dp4a_launch(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_
 
 }  // namespace
 
-// path: PIR_LWE_AUTO picks the tensor path from 8 queries up.
+// PIR_LWE_AUTO: which path is the faster one.  The CUDA cores stream the DB once per four
+// queries, at 5.5 TB/s with one or two queries, 4.2 with three, 3.4 with four; the tensor
+// cores once per 32, at 6.5, with about 4 us more of fixed cost (a second kernel and
+// scratch), and without the 2 us per query and K split that dp4a spends in its shortest
+// rows.  Measured: 16384 x 16384, one query 57.8 (dp4a) against 51.8 us, eight 163 against
+// 57; 1000 x 1024, four queries 16.5 against 13.0; 2000 x 512, 32 queries 10.4 against 13.2.
+bool tensor_path_wins(uint32_t D1, uint32_t D0, uint32_t B) {
+  const double mb = 1e-6 * D1 * D0, passes = (B + 3) / 4, tensor_passes = (B + 31) / 32;
+  const double gain_us = mb * ((B <= 2 ? 1 / 5.5 : B == 3 ? 1 / 4.2 : passes / 3.4) - tensor_passes / 6.5);
+  return gain_us >= 7 || (D0 >= 1024 && (B >= 4 || (B == 3 && gain_us >= 3)));
+}
+
+// The tensor path takes scratch for the query digits; where there is none left, or the
+// runtime offers no tensor maps, the CUDA cores answer.
 cudaError_t launch_lwe_gemm(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
-                            uint32_t path, cudaStream_t s) {
-  if (path == PIR_LWE_AUTO) path = B >= 8 ? PIR_LWE_TENSOR : PIR_LWE_SIMT;
-  if (path == PIR_LWE_TENSOR) return B >= 16 ? mma_launch<2>(A, D1, D0, Q, B, out, s) : mma_launch<1>(A, D1, D0, Q, B, out, s);
-  if (path == PIR_LWE_SIMT) {
-    uint32_t launches = 0;
-    if (B >= 4) return dp4a_launch<4>(A, D1, D0, Q, B, out, s, &launches);
-    if (B == 3) return dp4a_launch<3>(A, D1, D0, Q, B, out, s, &launches);
-    if (B == 2) return dp4a_launch<2>(A, D1, D0, Q, B, out, s, &launches);
-    return dp4a_launch<1>(A, D1, D0, Q, B, out, s, &launches);
+                            uint32_t path, cudaStream_t s, uint32_t *launches) {
+  if (path == PIR_LWE_AUTO) path = tensor_path_wins(D1, D0, B) ? PIR_LWE_TENSOR : PIR_LWE_SIMT;
+  if (path == PIR_LWE_TENSOR && tensor_maps_available()) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    keep_pool_memory(dev);  // scratch mapped anew after every synchronization costs 200 us a call
+    void *qt = nullptr;
+    e = cudaMallocAsync(&qt, lwe_tc_scratch_bytes(D0, B), s);
+    if (e == cudaSuccess) {
+      e = launch_lwe_tc(A, D1, D0, Q, B, out, static_cast<uint16_t *>(qt), s);
+      cudaFreeAsync(qt, s);
+      *launches = 2;
+      return e;
+    }
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
   }
-  return cudaErrorInvalidValue;
+  if (B >= 4) return dp4a_launch<4>(A, D1, D0, Q, B, out, s, launches);
+  if (B == 3) return dp4a_launch<3>(A, D1, D0, Q, B, out, s, launches);
+  if (B == 2) return dp4a_launch<2>(A, D1, D0, Q, B, out, s, launches);
+  return dp4a_launch<1>(A, D1, D0, Q, B, out, s, launches);
 }
 
 }  // namespace gbpir
@@ -310,8 +208,9 @@ extern "C" pir_status_t pir_lwe_answer(const int8_t *db, uint32_t D1, uint32_t D
   if (!db || !queries || !out || D1 == 0 || D0 == 0 || B == 0 || path > PIR_LWE_SIMT) return PIR_ERR_ARG;
   if (D0 % 16 != 0 || D0 > (1u << 24)) return PIR_ERR_ARG;
   if (((uintptr_t)db & 15u) || ((uintptr_t)queries & 15u) || ((uintptr_t)out & 15u)) return PIR_ERR_ARG;
-  cudaError_t e = launch_lwe_gemm(db, D1, D0, queries, B, out, path, static_cast<cudaStream_t>(stream));
+  uint32_t launches = 0;
+  cudaError_t e = launch_lwe_gemm(db, D1, D0, queries, B, out, path, static_cast<cudaStream_t>(stream), &launches);
   if (e != cudaSuccess) return cuda_status(e);
-  count_launches(1);
+  count_launches(launches);
   return PIR_OK;
 }

@@ -4,12 +4,18 @@
 #pragma once
 #include <cuda.h>  // CUtensorMap and its enums only: the encoder is reached through the runtime
 
+#include <cuda_fp16.h>
+
+#include <atomic>
 #include <cstdint>
 
 #include "async.cuh"
 
 namespace gbpir {
 namespace tcgen {
+
+constexpr uint32_t kSmemMax = 227u << 10;  // dynamic shared memory of one CTA
+constexpr uint32_t kSmemMin = 116u << 10;  // above half an SM's: one CTA per SM
 
 // Shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows x 16
 // bytes, `lbo` bytes between neighbours along K and `sbo` between 8-row groups.
@@ -139,6 +145,29 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// 32 columns of this warp's 32 lanes, a lane per thread.
+__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+      "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+// 16 columns of this warp's 32 lanes, a lane per thread.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+
 // 16 lanes x 16 columns, in the thread layout of tmem_st_16x256b_x4; complete only after
 // tmem_ld_wait.
 __device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t taddr, uint32_t (&r)[8]) {
@@ -177,6 +206,75 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+// The same of a 2-D box, on this CTA's barrier.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t c0, uint32_t c1, uint32_t bar,
+                                            uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar), "l"(policy)
+      : "memory");
+}
+
+// A ring position: slot and the parity of its current round.
+struct Ring {
+  uint32_t slot = 0, phase = 0;
+  __device__ __forceinline__ void next(uint32_t size) {
+    if (++slot == size) slot = 0, phase ^= 1;
+  }
+  __device__ __forceinline__ void skip(uint32_t count, uint32_t size) {
+    slot += count;
+    while (slot >= size) slot -= size, phase ^= 1;
+  }
+};
+
+// f16 pairs: bits - bias.
+__device__ __forceinline__ uint32_t half2_sub(uint32_t bits, uint32_t bias) {
+  const __half2 f = __hsub2(*reinterpret_cast<const __half2 *>(&bits), *reinterpret_cast<const __half2 *>(&bias));
+  return *reinterpret_cast<const uint32_t *>(&f);
+}
+
+// Launches a persistent kernel of one CTA (with CG = 2 a pair of CTAs) per SM (SM pair), no
+// more than there are units.  What the runtime says of the kernel on a device (how many
+// run at once, with any shared-memory size: one per SM) is asked once: the queries cost
+// more host time than the launch.
+template <auto Kernel, int CG, typename... A>
+cudaError_t launch_persistent(uint64_t units, uint32_t threads, size_t smem, cudaStream_t s, const A &...args) {
+  static std::atomic<int> known[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CG;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = CG == 2 ? 1 : 0;
+  int resident = known[dev].load(std::memory_order_acquire);
+  if (resident == 0) {
+    int sms = 0;
+    if ((e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax)) != cudaSuccess)
+      return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    resident = sms / CG;
+    cfg.gridDim = dim3((unsigned)(resident * CG), 1, 1);
+    if (CG == 2 && (cudaOccupancyMaxActiveClusters(&resident, Kernel, &cfg) != cudaSuccess || resident <= 0)) {
+      cudaGetLastError();  // clear the query's error: one cluster per SM pair
+      resident = sms / CG;
+    }
+    known[dev].store(resident, std::memory_order_release);
+  }
+  if ((uint64_t)resident > units) resident = (int)units;
+  cfg.gridDim = dim3((unsigned)(resident * CG), 1, 1);
+  return cudaLaunchKernelEx(&cfg, Kernel, args...);
+}
+
 }  // namespace tcgen
 
 // cuTensorMapEncodeTiled for a digit array [blocks][groups][128] of 16-bit elements (a
@@ -187,6 +285,9 @@ bool digit_tensor_map(CUtensorMap *map, const uint16_t *base, uint64_t groups, u
 // A u32 array [slots][rows][cols] with boxes of 32 columns x box_rows rows, 128-byte
 // swizzled; out-of-range elements read as zero.
 bool word_tensor_map(CUtensorMap *map, const uint32_t *base, uint64_t cols, uint64_t rows, uint64_t slots,
+                     uint32_t box_rows);
+// A byte array [rows][cols] with boxes of box_cols (<= 128) x box_rows, 128-byte swizzled.
+bool byte_tensor_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                      uint32_t box_rows);
 bool tensor_maps_available();
 

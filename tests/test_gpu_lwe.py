@@ -98,3 +98,24 @@ def test_arguments():
         with pytest.raises(g.PirError) as ei:
             g.pir_lwe_answer(*bad[:6], path=bad[6])
         assert ei.value.status == 1
+
+
+@pytest.mark.parametrize("D1,D0,B", [
+    (128, 128, 32),      # one row tile, one K stage
+    (129, 1024, 31),     # one row into a second tile of a pair, one whole chunk a tile
+    (385, 1040, 20),     # ragged pairs, one 16-byte tail past a chunk
+    (96, 4112, 33),      # K split over the CTAs, two tiles of queries
+    (2500, 16, 65),      # more tiles than CTAs of the shortest rows, three tiles of queries
+])
+def test_tensor_tile_edges(orc, D1, D0, B):
+    A, Q = rand(D1, D0, B, D1 * 3 + B)
+    assert np.array_equal(run(A, Q, g.PIR_LWE_TENSOR), orc.lwe_gemm(A, Q))
+    g.pir_check_device()
+
+
+def test_tensor_sums_at_the_f32_bound(orc):
+    """-128 times the digit -128 over whole 1024-byte sums: exactly 2^24 in every digit."""
+    D1, D0, B = 130, 2048, 5
+    A = np.full((D1, D0), -128, dtype=np.int8)
+    Q = np.full((B, D0), 0x7F7F7F80, dtype=np.uint32)  # digits -128, -128, -128, -128 mod 2^32
+    assert np.array_equal(run(A, Q, g.PIR_LWE_TENSOR), orc.lwe_gemm(A, Q))
