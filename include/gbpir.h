@@ -68,7 +68,9 @@ typedef enum {
                             u64), batches on the tensor cores (the words split into exact signed
                             base-256 f16 digits on the way, 1024-row f32 sums of at most 2^24);
                             tiles 1-8 keep a batch on the CUDA cores */
-  PIR_LAYOUT_LIMB = 1,   /* u8 limb planes [L*n slots][4][D2][D1]: INT8 tensor-pipe path    */
+  PIR_LAYOUT_LIMB = 1,   /* u8 limb planes [L*n slots][4][D2][D1]: the same tensor-core GEMM, the bytes
+                            as f16 (512-row f32 sums below 2^24); tiles 1-3 run it on the INT8
+                            tensor pipe (u8 x u8 -> s32)                                       */
   PIR_LAYOUT_TENSOR = 2  /* signed base-256 digits in bf16, 8 bytes per residue, laid out as
                             tensor-core operand tiles: the tcgen05 bf16 path (needs
                             D1 % 64 == 0 and D2 % 32 == 0)                                     */
@@ -135,7 +137,8 @@ typedef struct {
                         8 query rows (2B), 7 also D2 <= 512, 9 (the tensor-core GEMM,
                         the built-in choice for K-chunks of 128 rows and more) at
                         least 3; limb 2 and 3 need the
-                        rows padded to 16 to be multiples of 32 and 64; tensor 1 is
+                        rows padded to 16 to be multiples of 32 and 64 (limb 4, the
+                        f16 tensor-core GEMM, is the built-in choice); tensor 1 is
                         the 1-SM GEMM, 2 the CTA-pair (2-SM) GEMM, which needs
                         D2 % 64 == 0, 3 and 4 the 1-SM GEMM in clusters of 2 and 4
                         CTAs that multicast the query digits, which need D2 % 64

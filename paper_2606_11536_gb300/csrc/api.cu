@@ -227,19 +227,18 @@ uint32_t layout_chunk(int layout, uint32_t Kc) {
 size_t layout_qs_bytes(int layout, uint64_t nslots, uint32_t Kc, uint32_t Mp) {
   return (size_t)nslots * Kc * Mp * (layout == PIR_LAYOUT_TENSOR ? 8 : 4);
 }
-// The query copy of chunks of Kc rows under a tile choice: its bytes, and for the plain
-// layout's digit GEMM the rows of the pieces it takes a chunk in (else 0).  tight: within
-// the bytes that the other tiles take.
+// The query copy of chunks of Kc rows under a tile choice: its bytes, and for the digit GEMM
+// the rows of the pieces it takes a chunk in (else 0).  tight: within the bytes that the
+// other tiles take.
 struct QueryCopy {
   size_t bytes;
   uint32_t rows;
 };
-QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t Mp, uint32_t D2,
-                     bool tight) {
-  const size_t b = layout_qs_bytes(layout, nslots, Kc, Mp);
-  if (layout != PIR_LAYOUT_PLAIN || !gemm_plain_uses_digits(tile, M, Kc, D2)) return {b, 0};
-  const uint32_t rows = gemm_digit_rows(nslots, Kc, Mp, tight);
-  const size_t d = gemm_digit_query_bytes(nslots, rows, Mp);
+QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, bool tight) {
+  const size_t b = layout_qs_bytes(layout, nslots, Kc, layout_rows(layout, M));
+  if (!gemm_uses_digits(layout, tile, M, Kc)) return {b, 0};
+  const uint32_t rows = gemm_digit_rows(nslots, Kc, round4(M), tight);
+  const size_t d = gemm_digit_query_bytes(nslots, rows, round4(M));
   return {d > b ? d : b, rows};
 }
 uint32_t layout_tiles(int layout) {
@@ -345,7 +344,7 @@ struct StageTimer {
 
 // One K-chunk on the DB's GEMM path: the NTT-form chunk qhat [B][kc][2][L][n] to
 // the layout's query copy qs, then the GEMM accumulated into out [L*n][M][D2].
-// digit_rows: the plain layout's digit GEMM in pieces of so many rows (query_copy).
+// digit_rows: the digit GEMM in pieces of so many rows (query_copy).
 pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint32_t Mp, uint32_t i0, uint32_t kc,
                         uint32_t digit_rows, void *qs, uint32_t *out, uint32_t tile, int stall, StageTimer &tm,
                         cudaStream_t s) {
@@ -356,11 +355,10 @@ pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint
     for (uint32_t k0 = 0; k0 < kc; k0 += digit_rows) {
       const uint32_t kr = kc - k0 < digit_rows ? kc - k0 : digit_rows;
       tm.begin();
-      CK(launch_query_digits(c, qhat, B, kc, k0, kr, Mp, qt, s));
+      CK(launch_query_digits(c, db->layout, qhat, B, kc, k0, kr, round4(M), qt, s));
       tm.end(1, 1);
       tm.begin();
-      CK(launch_gemm_digit(c, static_cast<const uint32_t *>(db->resident), D1, D2, qt, M, Mp, i0 + k0, kr, out,
-                           i0 + k0 > 0, s));
+      CK(launch_gemm_digit(c, db->layout, db->resident, D1, D2, qt, M, round4(M), i0 + k0, kr, out, i0 + k0 > 0, s));
       tm.end(2, 1);
     }
     return PIR_OK;
@@ -457,7 +455,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   const size_t qhat_bytes = qhat_ready ? 0 : (size_t)B * Kc * 2 * L * n * 4;
   // (the stall test hook belongs to the TMA scan)
   const uint32_t qtile = stall ? 7 : o.tile;
-  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, Mp, D2, false);
+  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, false);
   const size_t out_bytes = nslots * M * D2 * 4;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   // Batch 1 on the TMA scan: the forward NTT writes the slot layout itself (pairs of
@@ -477,7 +475,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   cudaError_t ae = scratch.alloc(other_bytes + up(qc.bytes));
   if (ae == cudaErrorMemoryAllocation && qc.rows) {
     cudaGetLastError();
-    qc = query_copy(db->layout, qtile, nslots, Kc, M, Mp, D2, true);
+    qc = query_copy(db->layout, qtile, nslots, Kc, M, true);
     ae = scratch.alloc(other_bytes + up(qc.bytes));
   }
   CK(ae);
@@ -687,14 +685,14 @@ pir_status_t session_open(pir_db *db, uint32_t B, uint32_t kc_max, cudaStream_t 
   ses->o = o;
   ses->failed = PIR_OK;
   ses->qhat_bytes = (size_t)B * kc_max * ct * 4;
-  QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, Mp, p.D2, false);
+  QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, false);
   ses->stage_bytes = up(ses->qhat_bytes);
   const size_t out_bytes = nslots * M * p.D2 * 4;
   void *mem = nullptr;
   cudaError_t e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
   if (e == cudaErrorMemoryAllocation && qc.rows) {
     cudaGetLastError();
-    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, Mp, p.D2, true);
+    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, true);
     e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
   }
   ses->qs_bytes = qc.bytes;
@@ -1464,6 +1462,7 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
     for (uint32_t t = 4; t <= 6; ++t) tiles.push_back(t);
     if (scan_tma_supports(M, p.D2)) tiles.push_back(7);
   } else {
+    if (gemm_limb_tile_ok(kLimbDigitTile, Mp16)) tiles.push_back(kLimbDigitTile);
     tiles.push_back(1);
     if (Mp16 % 32 == 0) tiles.push_back(2);
     if (Mp16 % 64 == 0) tiles.push_back(3);

@@ -169,24 +169,25 @@ size_t lwe_tc_scratch_bytes(uint32_t D0, uint32_t B);
 cudaError_t launch_lwe_tc(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
                           uint16_t *qt, cudaStream_t s);
 
-// gemm_digit.cu: the same contract on the tensor cores, the DB words split into digits
-// on the way (tile 9 of the plain layout).  Its query operand is f16 digits
-// (gemm_digit_query_bytes) made by launch_query_digits from ciphertexts k0 ..
-// k0 + Kc - 1 of qhat [B][Ks][2][L][n]; Mp a multiple of 4, Kc <= kDigitMaxRows.
-constexpr uint32_t kDigitTile = 9;
+// gemm_digit.cu: the same contract on the tensor cores for the plain and limb layouts, the
+// DB residues split into digits on the way (tile 9 of the plain layout, 4 of the limb
+// layout).  Its query operand is f16 digits (gemm_digit_query_bytes) made by
+// launch_query_digits from ciphertexts k0 .. k0 + Kc - 1 of qhat [B][Ks][2][L][n]; Mp a
+// multiple of 4 (on either layout), Kc <= kDigitMaxRows.
+constexpr uint32_t kDigitTile = 9, kLimbDigitTile = 4;
 constexpr uint32_t kDigitMaxRows = 8192;
 bool gemm_digit_available();
 size_t gemm_digit_query_bytes(uint64_t nslots, uint32_t Kc, uint32_t Mp);
-cudaError_t launch_query_digits(const ParamCtx &c, const uint32_t *qhat, uint32_t B, uint32_t Ks, uint32_t k0,
-                                uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s);
-cudaError_t launch_gemm_digit(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint16_t *qt,
-                              uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
-                              cudaStream_t s);
+cudaError_t launch_query_digits(const ParamCtx &c, int layout, const uint32_t *qhat, uint32_t B, uint32_t Ks,
+                                uint32_t k0, uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s);
+cudaError_t launch_gemm_digit(const ParamCtx &c, int layout, const void *db, uint32_t D1, uint32_t D2,
+                              const uint16_t *qt, uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out,
+                              int acc, cudaStream_t s);
 // Rows of one digit GEMM of a chunk of Kc rows.  Its query digits take 8 bytes per
-// residue where the other plain tiles' query copy takes 4.
+// residue where the other tiles' query copy takes 4.
 uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight);
-// Whether the plain layout's tile choice for chunks of Kc rows is the digit GEMM.
-bool gemm_plain_uses_digits(uint32_t tile, uint32_t M, uint32_t Kc, uint32_t D2);
+// Whether a layout's tile choice for chunks of Kc rows is the digit GEMM.
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t Kc);
 
 // scan_tma.cu: the same contract for M <= 8 rows and D2 <= 512 (D2 % 4 == 0), as a
 // TMA-staged stream; stall_test makes its consumers wait on a barrier that never

@@ -1,5 +1,5 @@
-// gemm_digit.cu -- the batched first-dimension modular GEMM of the plain layout on the
-// tensor cores: the resident u32 residues are split into digits on the way to the MMA.
+// gemm_digit.cu -- the batched first-dimension modular GEMM of the plain and limb layouts
+// on the tensor cores: the resident residues are split into digits on the way to the MMA.
 //
 //   out[s][m][c] = sum_{i < Kc} qs[s][i][m] * db[s][i0 + i][c]   (mod q_j),  s = j*n + k
 //
@@ -13,6 +13,10 @@
 // Every 1024 rows the epilogue reads P back, weights digit pair (l, a) with
 // 2^(8 (l + a)) mod q, sums in int64 and keeps the sum in registers across the chunks;
 // it reduces mod q once per output.
+//
+// The limb layout's residues are their four bytes already, digits in [0, 255]: a byte under
+// the exponent of 1024, less 1024.  Its sums take 512 rows (512 * 255 * 128 < 2^24), and its
+// K positions are the rows in order.
 //
 // One MMA (M = 128 per CTA, N = 4 * query rows, K = 16) forms all 16 products.  A rows are
 // (DB column, digit) pairs, B rows (query row, digit) pairs n = 4 * m + a.  A lives in
@@ -37,12 +41,14 @@
 // how tcgen05.st.16x256b lays a thread's four words out.  Its K positions 4j .. 4j + 3 are
 // rows 2j, 2j + 1, 2j + 8, 2j + 9 of each 16 (the query digits are stored in that order),
 // so that the four row groups a warp reads at once fall into different swizzled chunks:
-// no bank conflicts.
+// no bank conflicts.  (LIMB: a block is 64 bytes of 128 (limb, column) rows, a lane reads its
+// own row, tcgen05.st.32x32b.)
 //
 // Measured (GB300, 2.07 GHz, against the CUDA-core tiles): 8 GiB DB (n = 4096, 2048 x 512),
 // batch 32: 69.4 -> 12.8 ms, 0.76 of the sustained bf16 rate as 16 digit products; 1 GiB DB
 // (n = 2048, 512 x 512), batch 8: 2.3 -> 0.83 ms, 5.2 TB/s of DB words; 1 GiB DB (n = 4096),
-// batch 4: 1.38 -> 0.73 ms.  With few query rows it is bound by HBM, from 2B = 32 by the
+// batch 4: 1.38 -> 0.73 ms; limb layout (n = 2048, 512 x 256), batch 32: 7.8 (INT8 mma.sync) ->
+// 1.4 ms.  With few query rows it is bound by HBM, from 2B = 32 by the
 // MMAs (and, where D1 is short, by the epilogue's serial parts).
 //
 // Every barrier wait is bounded; one that runs out sets the device error word.
@@ -50,7 +56,7 @@
 #include "common.cuh"
 #include "tcgen.cuh"
 
-#include <cuda_fp16.h>
+#include <type_traits>
 
 namespace gbpir {
 namespace {
@@ -68,7 +74,6 @@ constexpr uint32_t kThreads = (kMmaWarp + 1) * 32;
 constexpr uint32_t kRows = 64;                    // DB rows per block
 constexpr uint32_t kRawBytes = kRows * 32 * 4;    // one block of DB words
 constexpr uint32_t kBlockCols = kRows / 2;        // tensor-memory columns of one block's digits
-constexpr uint32_t kChunkRows = 1024;             // rows per exact f32 sum
 constexpr uint32_t kMaxRaw = 16, kMaxB = 4, kMaxA = 4;
 constexpr uint32_t kTmem = 512;
 constexpr uint32_t kBars = 2 * kMaxRaw + 2 * kMaxB + 2 * kMaxA + 2 * 3 + 1;
@@ -99,6 +104,13 @@ __device__ __forceinline__ int64_t mad_wide(int32_t x, int32_t y, int64_t acc) {
   return d;
 }
 
+__device__ __forceinline__ void ld_shared16(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+
 __device__ __forceinline__ uint32_t ld_shared(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
@@ -119,7 +131,7 @@ struct UnitWalk {
   }
 };
 
-template <int CG, int SUB>
+template <int CG, int SUB, bool LIMB>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_digit(DigArgs a, ModConst mc, const __grid_constant__ CUtensorMap tm_db,
                  const __grid_constant__ CUtensorMap tm_q) {
@@ -137,6 +149,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t rank = CG == 2 ? cluster_rank() : 0;
   const uint32_t first = blockIdx.x / CG, step = gridDim.x / CG;
   constexpr uint32_t kStageRows = SUB * kRows, H = 2 / SUB;
+  constexpr uint32_t kChunkRows = LIMB ? 512 : 1024;  // rows per exact f32 sum
   constexpr uint32_t kSets = 2 * H, kEpi = 4 * kSets, kCvt = kWorkers - kEpi, kGroups = kCvt / 4;
   constexpr int kPer = H == 1 ? 6 : 2, kItems = H * kPer;  // accumulator groups per epilogue set: a half's, a unit's
   const uint32_t nks = (a.Kc + kStageRows - 1) / kStageRows;  // stages of a tile per unit
@@ -182,8 +195,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---------------- converters ----------------
     const uint32_t quarter = warp & 3, group = (warp - kEpi) >> 2;
     const uint32_t rho = lane >> 2, j = lane & 3, ch = 2 * quarter + (rho >> 2);
-    const uint32_t off0 = 2 * j * 128 + ((ch ^ (2 * j)) << 4) + (rho & 3) * 4;
-    const uint32_t off1 = (2 * j + 1) * 128 + ((ch ^ (2 * j + 1)) << 4) + (rho & 3) * 4;
+    // LIMB: this lane's row and the swizzle of its 16-byte chunks; else the words of the
+    // even and the odd rows
+    const uint32_t lrow = 32 * (lane >> 3) + 8 * quarter + (lane & 7);
+    const uint32_t off0 = LIMB ? lrow * 64 : 2 * j * 128 + ((ch ^ (2 * j)) << 4) + (rho & 3) * 4;
+    const uint32_t off1 = LIMB ? (lrow >> 1 & 3) << 4
+                               : (2 * j + 1) * 128 + ((ch ^ (2 * j + 1)) << 4) + (rho & 3) * 4;
     const uint32_t bias = 0x64806480u, bias3 = 0x64006480u;  // f16 1152 | 1152 and 1152 | 1024
     const uint32_t ta = tmem + a.a0 + ((32 * quarter) << 16);
     const uint32_t fullA_lead = CG == 2 ? map_to_rank(fullA, 0) : fullA;
@@ -203,22 +220,35 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         const uint32_t base = raw0 + rr.slot * kRawBytes;
-        uint32_t lo[16], hi[16];  // digits 0, 1 and 2, 3 of this thread's column
+        uint32_t f[32];  // LIMB: this lane's 64 digits; else digits 0, 1 and 2, 3 of its column
+        if constexpr (LIMB) {
 #pragma unroll
-        for (int kb = 0; kb < 4; ++kb) {
-          uint32_t e[4], o[4];
+          for (int c = 0; c < 4; ++c) {
+            uint32_t x[4];
+            ld_shared16(base + off0 + ((c << 4) ^ off1), x);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const uint32_t y = ld_shared(base + (t & 1 ? off1 : off0) + (t >> 1) * 1024 + kb * 2048) + 0x00808080u;
-            e[t] = half2_sub((y & 0x00FF00FFu) | 0x64006400u, bias);
-            o[t] = half2_sub(__byte_perm(y, 0x64646464u, 0x4341), bias3);
+            for (int i = 0; i < 4; ++i) {
+              f[8 * c + 2 * i] = half2_sub(__byte_perm(x[i], 0x64646464u, 0x4140), 0x64006400u);
+              f[8 * c + 2 * i + 1] = half2_sub(__byte_perm(x[i], 0x64646464u, 0x4342), 0x64006400u);
+            }
           }
+        } else {
 #pragma unroll
-          for (int v = 0; v < 2; ++v) {
-            lo[4 * kb + v] = __byte_perm(e[2 * v], e[2 * v + 1], 0x5410);
-            lo[4 * kb + 2 + v] = __byte_perm(o[2 * v], o[2 * v + 1], 0x5410);
-            hi[4 * kb + v] = __byte_perm(e[2 * v], e[2 * v + 1], 0x7632);
-            hi[4 * kb + 2 + v] = __byte_perm(o[2 * v], o[2 * v + 1], 0x7632);
+          for (int kb = 0; kb < 4; ++kb) {
+            uint32_t e[4], o[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const uint32_t y = ld_shared(base + (t & 1 ? off1 : off0) + (t >> 1) * 1024 + kb * 2048) + 0x00808080u;
+              e[t] = half2_sub((y & 0x00FF00FFu) | 0x64006400u, bias);
+              o[t] = half2_sub(__byte_perm(y, 0x64646464u, 0x4341), bias3);
+            }
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+              f[4 * kb + v] = __byte_perm(e[2 * v], e[2 * v + 1], 0x5410);
+              f[4 * kb + 2 + v] = __byte_perm(o[2 * v], o[2 * v + 1], 0x5410);
+              f[16 + 4 * kb + v] = __byte_perm(e[2 * v], e[2 * v + 1], 0x7632);
+              f[16 + 4 * kb + 2 + v] = __byte_perm(o[2 * v], o[2 * v + 1], 0x7632);
+            }
           }
         }
         __syncwarp();
@@ -231,8 +261,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           fence_after();
         }
         const uint32_t dst = ta + (ra.slot * SUB + sub) * kBlockCols;
-        tmem_st_16x256b_x4(dst, lo);
-        tmem_st_16x256b_x4(dst + (16 << 16), hi);
+        if constexpr (LIMB) {
+          tmem_st_32x32b_x32(dst, f);
+        } else {
+          tmem_st_16x256b_x4(dst, f);
+          tmem_st_16x256b_x4(dst + (16 << 16), f + 16);
+        }
       }
       if (!ok) break;
       tmem_st_wait();
@@ -270,8 +304,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               break;
             }
             mbar_expect_tx(fullR + 8 * r.slot, kRawBytes);
-            tma_load_3d<1>(raw0 + r.slot * kRawBytes, &tm_db, c0 + t / SUB * 32,
-                           a.i0 + ks * kStageRows + t % SUB * kRows, w.s, fullR + 8 * r.slot, pol);
+            const uint32_t c = c0 + t / SUB * 32, i = a.i0 + ks * kStageRows + t % SUB * kRows;
+            if (LIMB)
+              tma_load_4d(raw0 + r.slot * kRawBytes, &tm_db, i, c, 0, w.s, fullR + 8 * r.slot, pol);
+            else
+              tma_load_3d<1>(raw0 + r.slot * kRawBytes, &tm_db, c, i, w.s, fullR + 8 * r.slot, pol);
           }
       }
       // never leave with copies in flight
@@ -469,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                  wgt[l + d], x);
                 sum[v] = x;
               }
-              // 16 products of 2^24 * 2^30 a chunk: below 2^62 after 8 chunks
+              // 16 products of 2^24 * 2^30 a chunk: below 2^62 after 16 chunks
               tot[it + g2] += (p ? sum[1] : sum[0]) + __shfl_xor_sync(0xffffffffu, p ? sum[0] : sum[1], 1);
             }
           }
@@ -515,14 +552,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 // qhat rows [B][Ks][2][L][n], ciphertexts k0 .. k0 + Kc - 1 of every query -> f16 digits
 // qt [s][u = i / 16][4 * Mp rows][16] in core-matrix blocks (element (row r, position k)
 // of a block at (r / 8) * 128 + (k / 8) * 64 + (r % 8) * 8 + k % 8), row r = 4m + a.
-// Position k = 4j + t holds ciphertext 2j + t % 2 + 8 (t / 2) of the 16; rows m >= M and
-// the ciphertexts from Kc up to a multiple of 64 are zero.
+// Position k = 4j + t holds ciphertext 2j + t % 2 + 8 (t / 2) of the 16 (in_order: k); rows
+// m >= M and the ciphertexts from Kc up to a multiple of 64 are zero.
 // CTA = 32 slots x 16 ciphertexts x 8 query rows, as k_query_to_tensor: residues are
 // staged in shared memory with coalesced reads along the slots; then a thread takes
 // (slot, m, K half) and writes the four 16-byte digit rows of its 8 residues.
 __global__ void __launch_bounds__(256) k_query_digits(const uint32_t *__restrict__ qhat, uint32_t M, uint32_t Mp,
                                                       uint32_t Ks, uint32_t k0, uint32_t Kc, uint32_t L, uint32_t logn,
-                                                      uint16_t *__restrict__ qt) {
+                                                      int in_order, uint16_t *__restrict__ qt) {
   __shared__ uint32_t vals[16][8][33];
   const uint32_t n = 1u << logn;
   const uint32_t s0 = blockIdx.x * 32, u = blockIdx.y, mb = blockIdx.z;
@@ -550,7 +587,7 @@ __global__ void __launch_bounds__(256) k_query_digits(const uint32_t *__restrict
     uint32_t b[8];  // 128 + signed digit in bytes 0..2, the top digit in byte 3
 #pragma unroll
     for (int e = 0; e < 8; ++e)  // position 8h + e: j = 2h + e / 4, t = e % 4
-      b[e] = vals[2 * (2 * h + e / 4) + (e & 1) + 8 * ((e >> 1) & 1)][ml][sl] + 0x00808080u;
+      b[e] = vals[in_order ? 8 * h + e : 2 * (2 * h + e / 4) + (e & 1) + 8 * ((e >> 1) & 1)][ml][sl] + 0x00808080u;
     const uint64_t s = s0 + sl;
     uint16_t *dst = qt + (s * Uc + u) * (uint64_t)Ntot * 16 + (4 * mb + (ml >> 1)) * 128 + h * 64 + (ml & 1) * 32;
 #pragma unroll
@@ -583,13 +620,18 @@ uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight) 
   return r < 64 ? 64 : r > kDigitMaxRows ? kDigitMaxRows : r;
 }
 
-bool gemm_plain_uses_digits(uint32_t tile, uint32_t M, uint32_t Kc, uint32_t D2) {
-  if (tile == kDigitTile) return true;
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t Kc) {
+  if (layout == PIR_LAYOUT_TENSOR) return false;
+  if (tile == (layout == PIR_LAYOUT_PLAIN ? kDigitTile : kLimbDigitTile)) return true;
+  if (tile != 0 || !gemm_digit_available()) return false;
+  // INT8 mma.sync at its peak is 1.3 to 7 times slower at every size measured (32 to 512 rows
+  // and columns, 1 to 32 queries).
+  if (layout == PIR_LAYOUT_LIMB) return true;
   // One query streams the DB at HBM speed on the CUDA cores already.  From 128 rows on the
   // digit GEMM wins at every width (1.2x at 512 columns and batch 4, up to 4x); at 64 rows
   // it still wins at 32 columns (1.5-3x) but loses at 256 (0.78-1.06x), where its
   // epilogue outweighs the products.
-  return tile == 0 && M >= 3 && Kc >= 128 && gemm_digit_available();
+  return M >= 3 && Kc >= 128;
 }
 
 bool gemm_digit_available() { return tensor_maps_available(); }
@@ -598,16 +640,16 @@ size_t gemm_digit_query_bytes(uint64_t nslots, uint32_t Kc, uint32_t Mp) {
   return (size_t)nslots * round64(Kc) * Mp * 8;
 }
 
-cudaError_t launch_query_digits(const ParamCtx &c, const uint32_t *qhat, uint32_t B, uint32_t Ks, uint32_t k0,
-                                uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s) {
+cudaError_t launch_query_digits(const ParamCtx &c, int layout, const uint32_t *qhat, uint32_t B, uint32_t Ks,
+                                uint32_t k0, uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s) {
   if (Mp % 4 != 0 || Kc == 0) return cudaErrorInvalidValue;
   dim3 grid((c.p.L << c.logn) / 32, round64(Kc) / 16, (Mp + 7) / 8);
-  k_query_digits<<<grid, 256, 0, s>>>(qhat, 2 * B, Mp, Ks, k0, Kc, c.p.L, c.logn, qt);
+  k_query_digits<<<grid, 256, 0, s>>>(qhat, 2 * B, Mp, Ks, k0, Kc, c.p.L, c.logn, layout == PIR_LAYOUT_LIMB, qt);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm_digit(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint16_t *qt,
-                              uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
+cudaError_t launch_gemm_digit(const ParamCtx &c, int layout, const void *db, uint32_t D1, uint32_t D2,
+                              const uint16_t *qt, uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
                               cudaStream_t s) {
   if (Kc == 0 || Kc > kDigitMaxRows || i0 + (uint64_t)Kc > D1 || Mp % 4 != 0 || Mp < M || D2 % 4 != 0)
     return cudaErrorInvalidValue;
@@ -651,12 +693,17 @@ cudaError_t launch_gemm_digit(const ParamCtx &c, const uint32_t *db, uint32_t D1
   size_t smem = a.SR * kRawBytes + a.SB * a.bstage + fixed;
   if (smem < kSmemMin) smem = kSmemMin;
   alignas(64) CUtensorMap tm_db = {}, tm_q = {};
-  if (!word_tensor_map(&tm_db, db, D2, D1, nslots, kRows) ||
+  const bool limb = layout == PIR_LAYOUT_LIMB;
+  if (!(limb ? limb_tensor_map(&tm_db, db, D1, D2, nslots, kRows) : word_tensor_map(&tm_db, db, D2, D1, nslots, kRows)) ||
       !digit_tensor_map(&tm_q, qt, Ntot / 8, nslots * a.Uc, a.NH / CG / 8, SUB * kRows / 16))
     return cudaErrorInvalidValue;
-  if (H == 2) return launch_persistent<k_gemm_digit<2, 1>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
-  return CG == 2 ? launch_persistent<k_gemm_digit<2, 2>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q)
-                 : launch_persistent<k_gemm_digit<1, 2>, 1>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
+  auto launch = [&](auto which) {
+    constexpr bool LIMB = decltype(which)::value;
+    if (H == 2) return launch_persistent<k_gemm_digit<2, 1, LIMB>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
+    if (CG == 2) return launch_persistent<k_gemm_digit<2, 2, LIMB>, 2>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
+    return launch_persistent<k_gemm_digit<1, 2, LIMB>, 1>(nunits, kThreads, smem, s, a, c.mod, tm_db, tm_q);
+  };
+  return limb ? launch(std::true_type()) : launch(std::false_type());
 }
 
 }  // namespace gbpir

@@ -188,8 +188,10 @@ cudaError_t limb_launch(const ParamCtx &c, const uint8_t *db, uint32_t D1, uint3
 }  // namespace
 
 // Tile ids: 1 = 16 x 128 (warps along columns), 2 = 32 x 64, 3 = 64 x 32 (warps along rows).
-// 0 picks by the padded row count Mp (a multiple of 16).
-uint32_t gemm_limb_tiles() { return 3; }
+// 4 = the f16 tensor-core GEMM (gemm_digit.cu), which takes another query operand and is
+// launched by its own entry point.  Where that does not apply, 0 picks by the padded row
+// count Mp (a multiple of 16).
+uint32_t gemm_limb_tiles() { return kLimbDigitTile; }
 
 bool gemm_limb_tile_ok(uint32_t tile, uint32_t Mp) {
   switch (tile) {
@@ -197,6 +199,7 @@ bool gemm_limb_tile_ok(uint32_t tile, uint32_t Mp) {
     case 1: return Mp % 16 == 0;
     case 2: return Mp % 32 == 0;
     case 3: return Mp % 64 == 0;
+    case kLimbDigitTile: return gemm_digit_available();
   }
   return false;
 }

@@ -893,7 +893,7 @@ bool digit_tensor_map(CUtensorMap *map, const uint16_t *base, uint64_t groups, u
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool word_tensor_map(CUtensorMap *map, const uint32_t *base, uint64_t cols, uint64_t rows, uint64_t slots,
+bool word_tensor_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t slots,
                      uint32_t box_rows) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
@@ -901,8 +901,21 @@ bool word_tensor_map(CUtensorMap *map, const uint32_t *base, uint64_t cols, uint
   const cuuint64_t strides[2] = {cols * 4, cols * rows * 4};
   const cuuint32_t box[3] = {32, box_rows, 1};
   const cuuint32_t estride[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t *>(base), dims, strides, box, estride,
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<void *>(base), dims, strides, box, estride,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool limb_tensor_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t slots,
+                     uint32_t box_rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return false;
+  const cuuint64_t dims[4] = {rows, cols, 4, slots};
+  const cuuint64_t strides[3] = {rows, rows * cols, rows * cols * 4};
+  const cuuint32_t box[4] = {box_rows, 32, 4, 1};
+  const cuuint32_t estride[4] = {1, 1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(base), dims, strides, box, estride,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -49,7 +49,7 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t d, uint32_t a, uint64_t b, u
 
 // 16 lanes x 32 columns: thread t holds rows t / 4 (registers 4v, 4v + 1) and t / 4 + 8
 // (4v + 2, 4v + 3) of columns 8v + 2 (t % 4) and the next one.
-__device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_t (&r)[16]) {
+__device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_t *r) {
   asm volatile(
       "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
           taddr),
@@ -216,6 +216,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       : "memory");
 }
 
+// A 4-D box, on this CTA's barrier.
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t c0, uint32_t c1, uint32_t c2,
+                                            uint32_t c3, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar), "l"(policy)
+      : "memory");
+}
+
 // A ring position: slot and the parity of its current round.
 struct Ring {
   uint32_t slot = 0, phase = 0;
@@ -284,8 +294,11 @@ bool digit_tensor_map(CUtensorMap *map, const uint16_t *base, uint64_t groups, u
                       uint32_t box_blocks);
 // A u32 array [slots][rows][cols] with boxes of 32 columns x box_rows rows, 128-byte
 // swizzled; out-of-range elements read as zero.
-bool word_tensor_map(CUtensorMap *map, const uint32_t *base, uint64_t cols, uint64_t rows, uint64_t slots,
+bool word_tensor_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t slots,
                      uint32_t box_rows);
+// Limb planes [slots][4][cols][rows] of bytes, boxes of box_rows (<= 64) bytes x 32 columns x
+// 4 limbs, 64-byte swizzled.
+bool limb_tensor_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t slots, uint32_t box_rows);
 // A byte array [rows][cols] with boxes of box_cols (<= 128) x box_rows, 128-byte swizzled.
 bool byte_tensor_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                      uint32_t box_rows);

@@ -1,6 +1,7 @@
-"""The plain layout's tensor-core GEMM over in-kernel digits (tile 9): equal, word for
-word, to the CUDA-core tiles and to the oracle at the edges of its tiles (64-row blocks,
-1024-row sums, 32-column tiles, accumulator widths from 16 to 256 columns)."""
+"""The tensor-core GEMM over in-kernel digits (tile 9 of the plain layout, 4 of the limb
+layout): equal, word for word, to the CUDA-core and INT8 tiles and to the oracle at the
+edges of its tiles (64-row blocks, 1024- and 512-row sums, 32-column tiles, accumulator
+widths from 16 to 256 columns)."""
 import numpy as np
 import pytest
 
@@ -13,13 +14,13 @@ pytestmark = pytest.mark.gpu
 DIGIT = 9
 
 
-def device_db(p, seed):
+def device_db(p, seed, layout=0):
     import torch
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
     nbytes = p.D1 * p.D2 * p.n * p.log2p // 8
     raw = torch.randint(0, 256, (nbytes,), generator=gen, dtype=torch.uint8, device="cuda")
-    return g.pir_setup_db(p, raw)
+    return g.pir_setup_db(p, raw, layout)
 
 
 def device_queries(p, B, seed):
@@ -63,16 +64,39 @@ def test_equals_the_cuda_core_tiles(D1, D2, L, batches):
         g.pir_free_db(db)
 
 
-def test_extreme_residues_and_the_oracle(orc):
+@pytest.mark.parametrize("D1,D2,L,batches", [
+    (32, 4, 2, (1, 2)),             # half a block of rows, one query
+    (96, 28, 1, (3, 12, 17)),       # a block and a half
+    (160, 36, 2, (1, 16, 24, 25)),  # two column tiles; 192 and 200 accumulator columns
+    (544, 68, 1, (4, 33)),          # 32 rows into a second 512-row sum; 256 + 8 rows
+    (1600, 32, 1, (1, 48, 65)),     # four sums; two and three tiles of query rows
+])
+def test_limb_layout_equals_the_int8_tiles(D1, D2, L, batches):
+    import torch
+    p = g.pir_make_params(2048, 8, D1, D2, L)
+    db = device_db(p, D1, layout=1)
+    try:
+        for B in batches:
+            q = device_queries(p, B, B)
+            ref = answer(db, q, B, tile=1)
+            assert torch.equal(answer(db, q, B, tile=4), ref), B
+            assert torch.equal(answer(db, q, B, tile=4, k_chunk=96), ref), B  # accumulated chunks
+            assert torch.equal(answer(db, q, B), ref), B
+    finally:
+        g.pir_free_db(db)
+
+
+@pytest.mark.parametrize("layout,tile", [(0, DIGIT), (1, 4)])
+def test_extreme_residues_and_the_oracle(orc, layout, tile):
     """Queries of q - 1 everywhere (the largest digits of every prime) and uniform ones."""
-    n, D1, D2, L, B = 2048, 136, 40, 2, 3
+    n, D1, D2, L, B = 2048, 160, 40, 2, 3
     p, P = g.pir_make_params(n, 16, D1, D2, L), orc.make_params(n, 16, D1, D2, L)
     raw = synth.raw_db(5, synth.raw_db_bytes(n, 16, D1, D2))
-    db = g.pir_setup_db(p, raw)
+    db = g.pir_setup_db(p, raw, layout)
     try:
         Q = random_queries(P, B, 6)
         Q[1] = np.array(P.qs, dtype=np.uint32)[None, None, :, None] - 1
-        R = from_dev(answer(db, to_dev(Q), B, tile=DIGIT), (B, D2, 2, L, n))
+        R = from_dev(answer(db, to_dev(Q), B, tile=tile), (B, D2, 2, L, n))
         assert np.array_equal(R, orc.answer(P, raw, Q))
     finally:
         g.pir_free_db(db)
