@@ -231,6 +231,24 @@ bool gemm_limb_tile_ok(uint32_t tile, uint32_t Mp);
 // Device helpers
 // ---------------------------------------------------------------------------
 
+// Division of n < 2^31 by a constant d (1 <= d < 2^31) known at launch, as one product:
+// with 2^(l-1) < d <= 2^l, floor(n / d) = floor(n M / 2^(31+l)) for M = ceil(2^(31+l) / d)
+// (Granlund and Montgomery, "Division by invariant integers using multiplication", PLDI
+// 1994).  A 64-bit division in a kernel is a subroutine of about a hundred instructions,
+// which every thread ran per row.
+struct FastDiv {
+  uint32_t d, mul, shift;
+  FastDiv() = default;
+  __host__ explicit FastDiv(uint64_t div) : d((uint32_t)div) {
+    uint32_t l = 0;
+    while ((1ull << l) < div) ++l;
+    mul = (uint32_t)(((1ull << (31 + l)) + div - 1) / div);
+    shift = 31 + l;
+  }
+  __device__ __forceinline__ uint32_t div(uint32_t n) const { return (uint32_t)(((uint64_t)n * mul) >> shift); }
+  __device__ __forceinline__ uint32_t mod(uint32_t n) const { return n - div(n) * d; }
+};
+
 // Shoup multiplication by a constant w < q with wsh = floor(w * 2^32 / q):
 // returns x * w mod q in [0, 2q) for any x < 2^32 (needs q < 2^31).
 __device__ __forceinline__ uint32_t shoup_mul(uint32_t x, uint32_t w, uint32_t wsh, uint32_t q) {

@@ -4,7 +4,10 @@
 // One CTA transforms one polynomial row of n residues (row r uses prime r % L).
 // Each thread holds 16 residues in registers and applies four butterfly stages
 // to them; the rows pass through shared memory (padded one word in sixteen) between
-// such radix-16 passes: n = 2^11 -> 4+4+3 bits, 2^12 -> 4+4+4, 2^13 -> 4+4+4+1.
+// such radix-16 passes: n = 2^11 -> 4+4+3 bits, 2^12 -> 4+4+4, 2^13 -> 4+4+4+1 (the last
+// bit between neighbouring threads, by shuffles).  Only the pass over the top bits mixes
+// elements of different warps: the others stay within blocks of n/16 elements that one
+// warp holds, so a row takes one block barrier and a warp barrier per further pass.
 //
 // Arithmetic: twiddles are psi^brv(i) (forward) and psi^-brv(i) (inverse) with
 // Shoup companions floor(w * 2^32 / q), so each twiddle product is one high and
@@ -15,30 +18,38 @@
 //
 // Output order: forward NTT(a)[k] = sum_t a_t psi^((2 brv(k) + 1) t), the natural
 // result of decimation in time with psi powers in bit-reversed order.
+//
+// Bound by the multiply-add pipe (a butterfly's high product and two low ones) and the
+// issue slots around it: 2 GiB of rows, n = 2^12, forward 1393 -> 1140 us (3.8 TB/s), n = 2^13,
+// inverse 1610 -> 1315 us, with row numbers divided by multiplication instead of 64-bit
+// divisions (a sixth of all instructions), one block barrier a row, whole-sector stores.
 #include "common.cuh"
 
 namespace gbpir {
 namespace {
 
-__device__ __forceinline__ uint32_t padx(uint32_t i) { return i + (i >> 4); }
+// Shared positions are padded: one word in sixteen, or for n = 2^13 two in thirty-two, which
+// is free of bank conflicts in every pass there (32 neighbours; 16 blocks of 32 by parity;
+// the first leaves one lane pair in two wavefronts where a warp takes 32 neighbours).
+template <int LOGN>
+__device__ __forceinline__ uint32_t padx(uint32_t i) {
+  return LOGN == 13 ? i + 2 * (i >> 5) : i + (i >> 4);
+}
 
-// Padded shared index of element e of a unit whose base index has bits
-// [BLO, BLO + RB) clear: when BLO >= 4, or BLO == 0 (a base aligned to 2^RB, RB <= 4),
-// the padding of base + e 2^BLO is that of base plus a constant, so the address is
-// the unit's padded base plus a compile-time offset.
-template <int BLO>
+// Padded position of element e of a unit whose base index has bits [BLO, BLO + 4) clear:
+// that of its base plus a constant where the padding adds up, so that the address is the
+// unit's plus a compile-time offset.
+template <int LOGN, int BLO>
 __device__ __forceinline__ uint32_t pidx(uint32_t pbase, uint32_t base, int e) {
-  if constexpr (BLO >= 4)
-    return pbase + (uint32_t)e * ((1u << BLO) + (1u << (BLO - 4)));
-  else if constexpr (BLO == 0)
-    return pbase + (uint32_t)e;
+  if constexpr (LOGN == 13 ? BLO <= 1 || BLO >= 5 : BLO == 0 || BLO >= 4)
+    return pbase + padx<LOGN>((uint32_t)e << BLO);
   else
-    return padx(base + ((uint32_t)e << BLO));
+    return padx<LOGN>(base + ((uint32_t)e << BLO));
 }
 
 // x - m if x >= m, else x (x < 2m <= 2^32): as unsigned values x - m wraps above x
-// exactly when x < m, so the minimum picks the right one in two integer operations.
-__device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m) { return min(x, x - m); }
+// exactly when x < m, so the minimum picks the right one: one add-and-minimum instruction.
+__device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m) { return __viaddmin_u32(x, 0u - m, x); }
 
 // Element j < L of a per-prime parameter array, by compare and select: indexing a
 // kernel parameter array with a run-time j makes the compiler copy the whole
@@ -51,18 +62,43 @@ __device__ __forceinline__ T pick(const T (&a)[PIR_MAX_L], uint32_t j) {
   return r;
 }
 
+// 32 bytes at once (a whole sector per thread; the address 32-byte aligned)
+__device__ __forceinline__ void ld_global32(const uint32_t *p, uint32_t *v) {
+  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void st_global32(uint32_t *p, const uint32_t *v) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+// 16 consecutive words of a row: rows start on 16-byte boundaries only
+__device__ __forceinline__ void load16(const uint32_t *__restrict__ p, uint32_t (&v)[16], bool wide) {
+  if (wide) {
+    ld_global32(p, v);
+    ld_global32(p + 8, v + 8);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 16; e += 4) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p + e));
+      v[e] = x.x, v[e + 1] = x.y, v[e + 2] = x.z, v[e + 3] = x.w;
+    }
+  }
+}
+__device__ __forceinline__ void store16(uint32_t *__restrict__ p, const uint32_t (&v)[16], bool wide) {
+  if (wide) {
+    st_global32(p, v);
+    st_global32(p + 8, v + 8);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 16; e += 4) *reinterpret_cast<uint4 *>(p + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+  }
+}
+__device__ __forceinline__ bool wide_ok(const void *p) { return ((uintptr_t)p & 31u) == 0; }
+
 // Source kinds of the first pass.
-enum { SRC_SMEM = 0, SRC_U32 = 1, SRC_RAW = 2 };
-
-// Destinations of a pass: shared memory (not the last pass), global memory
-// (canonical), a second shared buffer (canonical; the first row of a pair), or the
-// slot-major query layout as (first row, this row) pairs.
-enum { DST_SMEM = 0, DST_GLOBAL = 1, DST_PAIR = 2 };
-
-// (DST_PAIR parks a row's canonical results in its shared buffer; the pair kernel
-// then writes element k of rows (i, comp 0) and (i, comp 1) of prime j to
-// slots[((j*n + k) * Kc + i) * 2 + comp], the plain slot layout with Mp = 2.)
-struct SlotDst {};
+enum { SRC_U32 = 1, SRC_RAW = 2 };
 
 struct RawSrc {
   const uint8_t *raw;  // little-endian bit stream of log2p-bit coefficients
@@ -76,11 +112,19 @@ struct RawSrc {
   }
 };
 
-// Source rows of a launch: local row r reads row off + (r / G) * S + r % G, so a
-// chunk of ciphertexts can be taken out of every query of a batch without a copy.
-struct RowMap {  // local row r reads source row off + (r / G) * S + (r % G) * T
-  uint64_t off, G, S, T;
-  __device__ __forceinline__ uint64_t operator()(uint64_t r) const { return off + (r / G) * S + (r % G) * T; }
+// Source rows of a launch: local row r reads source row off + (r / G) * S + (r % G) * T, so
+// a chunk of ciphertexts can be taken out of every query of a batch without a copy.  Row
+// numbers stay below 2^31 (a row is 8 KiB at least).
+struct RowMap {
+  uint32_t off, S, T;
+  FastDiv G, L;  // L: the row's prime is r % L
+  RowMap() = default;
+  RowMap(uint64_t o, uint64_t g, uint64_t s, uint64_t t, uint32_t l)
+      : off((uint32_t)o), S((uint32_t)s), T((uint32_t)t), G(g), L(l) {}
+  __device__ __forceinline__ uint64_t operator()(uint32_t r) const {
+    const uint32_t g = G.div(r);
+    return off + (uint64_t)g * S + (r - g * G.d) * T;
+  }
 };
 
 // Coefficient `t` of plaintext polynomial `poly` from the raw bit stream.
@@ -132,8 +176,11 @@ __device__ __forceinline__ void fwd_bfly(uint32_t (&v)[1 << RB], const Pairs<CNT
       const uint32_t y = v[E | (1 << LB)];
       x = csub(x, q2);                                                              // [0, 2q)
       const uint32_t t = shoup_mul(y, p.template w<(E >> (LB + 1))>(), p.template ws<(E >> (LB + 1))>(), q);  // [0, 2q)
-      v[E] = x + t;                                                                 // [0, 4q)
-      v[E | (1 << LB)] = x - t + q2;                                                // (0, 4q)
+      // x - t + 2q as 2x + 2q - (x + t): two instructions either way, but in this form the
+      // compiler's butterfly issues in 3.9 cycles per warp against 5.8
+      const uint32_t s = x + t;
+      v[E] = s;                                                                     // [0, 4q)
+      v[E | (1 << LB)] = x + x + q2 - s;                                            // (0, 4q)
     }
     fwd_bfly<RB, LB, E + 1, CNT>(v, p, q);
   }
@@ -170,10 +217,9 @@ __device__ __forceinline__ void inv_bfly(uint32_t (&v)[1 << RB], const Pairs<CNT
     if constexpr ((E & (1 << LB)) == 0) {
       const uint32_t q2 = 2 * q;
       const uint32_t x = v[E], y = v[E | (1 << LB)];
-      uint32_t s = x + y;
-      s = csub(s, q2);
-      v[E] = s;
-      v[E | (1 << LB)] = shoup_mul(x - y + q2, p.template w<(E >> (LB + 1))>(), p.template ws<(E >> (LB + 1))>(), q);
+      const uint32_t s = x + y;
+      v[E] = csub(s, q2);
+      v[E | (1 << LB)] = shoup_mul(x + x + q2 - s, p.template w<(E >> (LB + 1))>(), p.template ws<(E >> (LB + 1))>(), q);
     }
     inv_bfly<RB, LB, E + 1, CNT>(v, p, q);
   }
@@ -203,151 +249,190 @@ __device__ __forceinline__ void inv_stages(uint32_t (&v)[1 << RB], uint32_t hi, 
   if constexpr (LB < RB - 1) inv_stages<RB, BLO, LOGN, LB + 1>(v, hi, tw, q);
 }
 
-// One radix-2^RB pass over the whole row: unit u holds the 2^RB elements whose
-// index has bits [BLO, BLO+RB) free and the rest fixed by u.
-template <int LOGN, int RB, int BLO, bool FWD, int SRC, int DST>
-__device__ __forceinline__ void ntt_pass(uint32_t *sm, const uint32_t *__restrict__ gin, const RawSrc &rs,
-                                         uint64_t poly, uint32_t *__restrict__ gout, const uint2 *__restrict__ tw,
-                                         uint32_t q, uint32_t ninv,
-                                         uint32_t ninv_sh, const SlotDst *sd = nullptr,
-                                         uint32_t tid = threadIdx.x) {
-  constexpr int N = 1 << LOGN, T = N / 16, UNITS = N >> RB, PER = UNITS / T;
-  static_assert(UNITS % T == 0, "pass plan");
+// The passes of one row by T = n/16 threads, 16 residues v each.  sm is the row's shared
+// buffer (padded).
+
+// Forward, bits LOGN - 1 .. LOGN - 4 (the input from global memory), into shared memory.
+template <int LOGN, int SRC>
+__device__ __forceinline__ void fwd_first(uint32_t *sm, const uint32_t *__restrict__ gin, const RawSrc &rs,
+                                          uint64_t poly, const uint2 *__restrict__ tw, uint32_t q, uint32_t tid) {
+  constexpr int BLO = LOGN - 4;
+  uint32_t v[16];
 #pragma unroll
-  for (int r = 0; r < PER; ++r) {
-    const uint32_t u = tid + r * T;
-    const uint32_t lo = u & ((1u << BLO) - 1), hi = u >> BLO;
-    const uint32_t base = (hi << (BLO + RB)) | lo;
-    const uint32_t pbase = padx(base);
-    uint32_t v[1 << RB];
-    if constexpr (SRC == SRC_U32 && BLO == 0 && RB >= 2) {
+  for (int e = 0; e < 16; ++e) {
+    const uint32_t idx = tid + ((uint32_t)e << BLO);
+    v[e] = SRC == SRC_U32 ? __ldg(gin + idx) : raw_coeff(rs, poly, idx, LOGN);
+  }
+  fwd_stages<4, BLO, LOGN>(v, 0, tw, q);
+  const uint32_t pbase = padx<LOGN>(tid);
 #pragma unroll
-      for (int e = 0; e < (1 << RB); e += 4) {
-        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(gin + base + e));
-        v[e] = x.x, v[e + 1] = x.y, v[e + 2] = x.z, v[e + 3] = x.w;
-      }
+  for (int e = 0; e < 16; ++e) sm[pidx<LOGN, BLO>(pbase, tid, e)] = v[e];
+}
+
+// A radix-16 pass on bits BLO .. BLO + 3, shared memory to shared memory.
+template <int LOGN, int BLO, bool FWD>
+__device__ __forceinline__ void mid_pass(uint32_t *sm, const uint2 *__restrict__ tw, uint32_t q, uint32_t tid) {
+  const uint32_t lo = tid & ((1u << BLO) - 1), hi = tid >> BLO, base = (hi << (BLO + 4)) | lo, pbase = padx<LOGN>(base);
+  uint32_t v[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) v[e] = sm[pidx<LOGN, BLO>(pbase, base, e)];
+  if constexpr (FWD)
+    fwd_stages<4, BLO, LOGN>(v, hi, tw, q);
+  else
+    inv_stages<4, BLO, LOGN>(v, hi, tw, q);
+#pragma unroll
+  for (int e = 0; e < 16; ++e) sm[pidx<LOGN, BLO>(pbase, base, e)] = v[e];
+}
+
+// The 8 twiddle pairs of bit 0 for elements 16 tid .. 16 tid + 15 (the lane-major copy).
+template <int LOGN>
+__device__ __forceinline__ void bit0_twiddles(Pairs<8> &p, const uint2 *__restrict__ tw, uint32_t tid) {
+  p.load_lane_major(reinterpret_cast<const uint4 *>(tw + (1u << LOGN)) + tid, 1u << (LOGN - 4));
+}
+
+// Forward, the bits below; v becomes elements 16 tid .. 16 tid + 15 of the result, canonical.
+// n = 2^13: bits 4..1 give thread tid the elements of one parity of 32 consecutive ones;
+// neighbours trade halves and take the pairs of bit 0.
+template <int LOGN>
+__device__ __forceinline__ void fwd_last(const uint32_t *sm, const uint2 *__restrict__ tw, uint32_t q, uint32_t tid,
+                                         uint32_t (&v)[16]) {
+  if constexpr (LOGN == 13) {
+    const uint32_t lo = tid & 1, hi = tid >> 1, base = (hi << 5) | lo, pbase = padx<LOGN>(base);
+    uint32_t w[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) w[e] = sm[pidx<LOGN, 1>(pbase, base, e)];
+    fwd_stages<4, 1, LOGN>(w, hi, tw, q);
+    Pairs<8> p;
+    bit0_twiddles<LOGN>(p, tw, tid);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, lo ? w[i] : w[i + 8], 1);
+      v[2 * i] = lo ? got : w[i];
+      v[2 * i + 1] = lo ? w[i + 8] : got;
+    }
+    fwd_bfly<4, 0, 0, 8>(v, p, q);
+  } else {
+    const uint32_t pbase = padx<LOGN>(16 * tid);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = sm[pbase + e];
+    if constexpr (LOGN == 12) {
+      fwd_stages<4, 0, LOGN>(v, tid, tw, q);
     } else {
 #pragma unroll
-      for (int e = 0; e < (1 << RB); ++e) {
-        const uint32_t idx = base + ((uint32_t)e << BLO);
-        if constexpr (SRC == SRC_SMEM)
-          v[e] = sm[pidx<BLO>(pbase, base, e)];
-        else if constexpr (SRC == SRC_U32)
-          v[e] = __ldg(gin + idx);
-        else
-          v[e] = raw_coeff(rs, poly, idx, LOGN);
+      for (int r = 0; r < 2; ++r) {
+        uint32_t w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = v[8 * r + e];
+        fwd_stages<3, 0, LOGN>(w, 2 * tid + r, tw, q);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[8 * r + e] = w[e];
       }
     }
-    if constexpr (FWD)
-      fwd_stages<RB, BLO, LOGN>(v, hi, tw, q);
-    else
-      inv_stages<RB, BLO, LOGN>(v, hi, tw, q);
-    if constexpr (DST != DST_SMEM) {
+  }
 #pragma unroll
-      for (int e = 0; e < (1 << RB); ++e) {
-        uint32_t x = v[e];
-        if constexpr (FWD) {
-          x = csub(x, 2 * q);
-          x = csub(x, q);
-        } else {
-          x = shoup_mul(x, ninv, ninv_sh, q);
-          x = csub(x, q);
-        }
-        v[e] = x;
-      }
-      if constexpr (DST == DST_PAIR) {
+  for (int e = 0; e < 16; ++e) v[e] = csub(csub(v[e], 2 * q), q);
+}
+
+// The forward transform of one row; v as fwd_last leaves it.
+template <int LOGN, int SRC>
+__device__ __forceinline__ void fwd_row(uint32_t *sm, const uint32_t *__restrict__ gin, const RawSrc &rs, uint64_t poly,
+                                        const uint2 *__restrict__ tw, uint32_t q, uint32_t tid, uint32_t (&v)[16]) {
+  fwd_first<LOGN, SRC>(sm, gin, rs, poly, tw, q, tid);
+  __syncthreads();
+  mid_pass<LOGN, LOGN - 8, true>(sm, tw, q, tid);
+  __syncwarp();
+  fwd_last<LOGN>(sm, tw, q, tid, v);
+}
+
+// Inverse, bits 0 .. 3 (n = 2^13: 0 .. 4) of elements 16 tid .. 16 tid + 15 in v, into shared
+// memory.
+template <int LOGN>
+__device__ __forceinline__ void inv_first(uint32_t *sm, const uint2 *__restrict__ tw, uint32_t q, uint32_t tid,
+                                          uint32_t (&v)[16]) {
+  if constexpr (LOGN == 13) {
+    const uint32_t lo = tid & 1, hi = tid >> 1, base = (hi << 5) | lo, pbase = padx<LOGN>(base);
+    Pairs<8> p;
+    bit0_twiddles<LOGN>(p, tw, tid);
+    inv_bfly<4, 0, 0, 8>(v, p, q);
+    uint32_t w[16];
 #pragma unroll
-        for (int e = 0; e < (1 << RB); ++e) sm[pidx<BLO>(pbase, base, e)] = v[e];
-      } else if constexpr (BLO == 0 && RB >= 2) {
-#pragma unroll
-        for (int e = 0; e < (1 << RB); e += 4)
-          *reinterpret_cast<uint4 *>(gout + base + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-      } else if constexpr (BLO == 0 && RB == 1) {
-        *reinterpret_cast<uint2 *>(gout + base) = make_uint2(v[0], v[1]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < (1 << RB); ++e) gout[base + ((uint32_t)e << BLO)] = v[e];
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < (1 << RB); ++e) sm[pidx<BLO>(pbase, base, e)] = v[e];
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, lo ? v[2 * i] : v[2 * i + 1], 1);
+      w[i] = lo ? got : v[2 * i];
+      w[i + 8] = lo ? v[2 * i + 1] : got;
     }
+    inv_stages<4, 1, LOGN>(w, hi, tw, q);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) sm[pidx<LOGN, 1>(pbase, base, e)] = w[e];
+  } else {
+    inv_stages<4, 0, LOGN>(v, tid, tw, q);
+    const uint32_t pbase = padx<LOGN>(16 * tid);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) sm[pbase + e] = v[e];
   }
 }
 
+// Inverse, the top bits, times n^-1, canonical; element idx goes to out(idx, value).
+template <int LOGN, typename Out>
+__device__ __forceinline__ void inv_last(const uint32_t *sm, const uint2 *__restrict__ tw, uint32_t q, uint32_t ninv,
+                                         uint32_t ninv_sh, uint32_t tid, Out out) {
+  constexpr int RB = LOGN == 11 ? 3 : 4, BLO = LOGN - RB, PER = 16 >> RB, T = 1 << (LOGN - 4);
+#pragma unroll
+  for (int r = 0; r < PER; ++r) {
+    const uint32_t lo = tid + r * T, pbase = padx<LOGN>(lo);
+    uint32_t v[1 << RB];
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e) v[e] = sm[pidx<LOGN, BLO>(pbase, lo, e)];
+    inv_stages<RB, BLO, LOGN>(v, 0, tw, q);
+#pragma unroll
+    for (int e = 0; e < (1 << RB); ++e)
+      out(lo + ((uint32_t)e << BLO), csub(shoup_mul(v[e], ninv, ninv_sh, q), q));
+  }
+}
+
+// CTAs per SM: 1280 threads for n = 2^11 and 2^12 (48 registers), 1536 for 2^13 (40; with two
+// CTAs of 512 the inverse took 1562 instead of 1315 us on 2 GiB).
+template <int LOGN>
+constexpr int kNttCtas = LOGN == 13 ? 3 : 20480 >> LOGN;
+
 template <int LOGN, int SRC>
-__global__ void __launch_bounds__((1 << LOGN) / 16, 20480 >> LOGN)  // >= 1280 threads per SM (measured fastest)
+__global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
     k_ntt_fwd(const uint32_t *__restrict__ src, RowMap rm, RawSrc rs, uint32_t *__restrict__ dst, NttConst C,
-              uint32_t L, uint64_t rows) {
+              uint32_t rows) {
   constexpr int N = 1 << LOGN;
   extern __shared__ uint32_t sm[];
-  for (uint64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const uint32_t j = (uint32_t)(row % L);
-    const uint32_t q = pick(C.q, j);
-    const uint2 *tw = pick(C.fwd, j);
-    const uint32_t *gin = src ? src + rm(row) * N : nullptr;
-    uint32_t *gout = dst + row * N;
-    const uint64_t poly = SRC == SRC_RAW ? rs.poly(row / L) : 0;
-    if constexpr (LOGN == 11) {
-      ntt_pass<11, 4, 7, true, SRC, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<11, 4, 3, true, SRC_SMEM, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<11, 3, 0, true, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-    } else if constexpr (LOGN == 12) {
-      ntt_pass<12, 4, 8, true, SRC, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<12, 4, 4, true, SRC_SMEM, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<12, 4, 0, true, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-    } else {
-      ntt_pass<13, 4, 9, true, SRC, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<13, 4, 5, true, SRC_SMEM, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<13, 4, 1, true, SRC_SMEM, DST_SMEM>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-      __syncthreads();
-      ntt_pass<13, 1, 0, true, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, poly, gout, tw, q, 0, 0);
-    }
-    __syncthreads();  // the next row reuses shared memory
+  const bool wide = wide_ok(dst);
+  for (uint32_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    const uint32_t p = rm.L.div(row), j = row - p * rm.L.d;
+    const uint64_t poly = SRC == SRC_RAW ? rs.poly(p) : 0;
+    uint32_t v[16];
+    fwd_row<LOGN, SRC>(sm, SRC == SRC_U32 ? src + rm(row) * N : nullptr, rs, poly, pick(C.fwd, j), pick(C.q, j),
+                       threadIdx.x, v);
+    store16(dst + (uint64_t)row * N + 16 * threadIdx.x, v, wide);
+    if (row + gridDim.x < rows) __syncthreads();  // the next row reuses shared memory
   }
 }
 
 template <int LOGN>
-__global__ void __launch_bounds__((1 << LOGN) / 16, 20480 >> LOGN)  // >= 1280 threads per SM (measured fastest)
-    k_ntt_inv(const uint32_t *__restrict__ src, RowMap rm, uint32_t *__restrict__ dst, NttConst C, uint32_t L,
-              uint64_t rows) {
+__global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
+    k_ntt_inv(const uint32_t *__restrict__ src, RowMap rm, uint32_t *__restrict__ dst, NttConst C, uint32_t rows) {
   constexpr int N = 1 << LOGN;
   extern __shared__ uint32_t sm[];
-  const RawSrc rs = {};
-  for (uint64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const uint32_t j = (uint32_t)(row % L);
-    const uint32_t q = pick(C.q, j), ni = pick(C.ninv, j), nis = pick(C.ninv_sh, j);
+  const uint32_t tid = threadIdx.x;
+  const bool wide = wide_ok(src);
+  for (uint32_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    const uint32_t j = rm.L.mod(row);
+    const uint32_t q = pick(C.q, j);
     const uint2 *tw = pick(C.inv, j);
-    const uint32_t *gin = src + rm(row) * N;
-    uint32_t *gout = dst + row * N;
-    if constexpr (LOGN == 11) {
-      ntt_pass<11, 4, 0, false, SRC_U32, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<11, 4, 4, false, SRC_SMEM, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<11, 3, 8, false, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-    } else if constexpr (LOGN == 12) {
-      ntt_pass<12, 4, 0, false, SRC_U32, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<12, 4, 4, false, SRC_SMEM, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<12, 4, 8, false, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-    } else {
-      ntt_pass<13, 4, 0, false, SRC_U32, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<13, 4, 4, false, SRC_SMEM, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<13, 4, 8, false, SRC_SMEM, DST_SMEM>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-      __syncthreads();
-      ntt_pass<13, 1, 12, false, SRC_SMEM, DST_GLOBAL>(sm, gin, rs, 0, gout, tw, q, ni, nis);
-    }
+    uint32_t *gout = dst + (uint64_t)row * N;
+    uint32_t v[16];
+    load16(src + rm(row) * N + 16 * tid, v, wide);
+    inv_first<LOGN>(sm, tw, q, tid, v);
+    __syncwarp();
+    mid_pass<LOGN, LOGN == 13 ? 5 : 4, false>(sm, tw, q, tid);
     __syncthreads();
+    inv_last<LOGN>(sm, tw, q, pick(C.ninv, j), pick(C.ninv_sh, j), tid, [&](uint32_t i, uint32_t x) { gout[i] = x; });
+    if (row + gridDim.x < rows) __syncthreads();
   }
 }
 
@@ -402,48 +487,37 @@ __device__ __forceinline__ uint32_t switch_coeff(const uint32_t *sm, uint32_t pa
 // half h inverts rows h, h + 2, ... into their own shared buffers (canonical), then
 // all threads switch the coefficients, four per 16-byte store.
 template <int LOGN>
-__global__ void __launch_bounds__((1 << LOGN) / 8, 8192 >> LOGN)  // <= 64 registers: 1024 threads per SM
+__global__ void __launch_bounds__((1 << LOGN) / 8, LOGN == 13 ? 1 : 12288 >> LOGN)  // 1024 or 1536 threads per SM
     k_ntt_inv_switch(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst, NttConst C, SwitchConst W,
                      uint32_t L) {
   constexpr int N = 1 << LOGN, PADN = N + N / 16, T = N / 16;
   extern __shared__ uint32_t sm[];
   const uint32_t half = threadIdx.x / T, tid = threadIdx.x % T;
-  const RawSrc rs = {};
-  uint32_t *gout = nullptr;
+  const bool wide = wide_ok(src);
   for (uint32_t r = 0; r < (L + 1) / 2; ++r) {
     const uint32_t j = 2 * r + half;
     const bool act = j < L;  // the barriers below are reached by both halves
     const uint32_t jj = act ? j : 0;
     uint32_t *smh = sm + jj * PADN;
-    const uint32_t q = pick(C.q, jj), ni = pick(C.ninv, jj), nis = pick(C.ninv_sh, jj);
+    const uint32_t q = pick(C.q, jj);
     const uint2 *tw = pick(C.inv, jj);
-    const uint32_t *gin = src + ((uint64_t)blockIdx.x * L + jj) * N;
-    if constexpr (LOGN == 11) {
-      if (act) ntt_pass<11, 4, 0, false, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<11, 4, 4, false, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<11, 3, 8, false, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-    } else if constexpr (LOGN == 12) {
-      if (act) ntt_pass<12, 4, 0, false, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<12, 4, 4, false, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<12, 4, 8, false, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-    } else {
-      if (act) ntt_pass<13, 4, 0, false, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<13, 4, 4, false, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<13, 4, 8, false, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
-      __syncthreads();
-      if (act) ntt_pass<13, 1, 12, false, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, ni, nis, nullptr, tid);
+    if (act) {
+      uint32_t v[16];
+      load16(src + ((uint64_t)blockIdx.x * L + jj) * N + 16 * tid, v, wide);
+      inv_first<LOGN>(smh, tw, q, tid, v);
+      __syncwarp();
+      mid_pass<LOGN, LOGN == 13 ? 5 : 4, false>(smh, tw, q, tid);
     }
+    __syncthreads();
+    // (the last pass reads and writes the same elements of a thread)
+    if (act)
+      inv_last<LOGN>(smh, tw, q, pick(C.ninv, jj), pick(C.ninv_sh, jj), tid,
+                     [&](uint32_t i, uint32_t x) { smh[padx<LOGN>(i)] = x; });
     __syncthreads();
   }
   uint32_t *out = dst + (uint64_t)blockIdx.x * N;
   for (uint32_t g = threadIdx.x; g < (uint32_t)N / 4; g += blockDim.x) {
-    const uint32_t pt = padx(4 * g);  // four consecutive positions stay consecutive
+    const uint32_t pt = padx<LOGN>(4 * g);  // four consecutive positions stay consecutive
     uint4 y;
     y.x = switch_coeff(sm, PADN, pt + 0, C, W, L);
     y.y = switch_coeff(sm, PADN, pt + 1, C, W, L);
@@ -470,36 +544,19 @@ __global__ void __launch_bounds__((1 << LOGN) / 8)
   const uint32_t q = pick(C.q, j);
   const uint2 *tw = pick(C.fwd, j);
   const uint32_t *gin = src + (row0 + (uint64_t)i * 2 * L + (uint64_t)half * L + j) * N;
-  const RawSrc rs = {};
-  uint32_t *gout = nullptr;
-  if constexpr (LOGN == 11) {
-    ntt_pass<11, 4, 7, true, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<11, 4, 3, true, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<11, 3, 0, true, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-  } else if constexpr (LOGN == 12) {
-    ntt_pass<12, 4, 8, true, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<12, 4, 4, true, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<12, 4, 0, true, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-  } else {
-    ntt_pass<13, 4, 9, true, SRC_U32, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<13, 4, 5, true, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<13, 4, 1, true, SRC_SMEM, DST_SMEM>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-    __syncthreads();
-    ntt_pass<13, 1, 0, true, SRC_SMEM, DST_PAIR>(smh, gin, rs, 0, gout, tw, q, 0, 0, nullptr, tid);
-  }
+  uint32_t v[16];
+  fwd_row<LOGN, SRC_U32>(smh, gin, RawSrc{}, 0, tw, q, tid, v);
+  // n = 2^13 reads its neighbours' words in the last pass
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 16; ++e) smh[padx<LOGN>(16 * tid) + e] = v[e];
   __syncthreads();
   uint32_t *dst = slots + ((uint64_t)j * N * stride + col0 + i) * 2;
   for (uint32_t k = threadIdx.x; k < (uint32_t)N; k += 2 * T)
-    *reinterpret_cast<uint2 *>(dst + (uint64_t)k * stride * 2) = make_uint2(sm[padx(k)], sm[PADN + padx(k)]);
+    *reinterpret_cast<uint2 *>(dst + (uint64_t)k * stride * 2) = make_uint2(sm[padx<LOGN>(k)], sm[PADN + padx<LOGN>(k)]);
 }
 
-constexpr uint64_t kMaxGrid = 1u << 30;
+constexpr uint64_t kMaxGrid = 1u << 30, kMaxRows = 0x7fffffffull;
 
 template <int LOGN>
 cudaError_t fwd_launch(const ParamCtx &c, const uint32_t *src, const RowMap &rm, const RawSrc &rs, uint32_t *dst,
@@ -508,9 +565,9 @@ cudaError_t fwd_launch(const ParamCtx &c, const uint32_t *src, const RowMap &rm,
   const size_t smem = ((1u << LOGN) + (1u << LOGN) / 16) * sizeof(uint32_t);
   const unsigned grid = (unsigned)(rows < kMaxGrid ? rows : kMaxGrid);
   if (raw)
-    k_ntt_fwd<LOGN, SRC_RAW><<<grid, T, smem, s>>>(nullptr, rm, rs, dst, c.ntt, c.p.L, rows);
+    k_ntt_fwd<LOGN, SRC_RAW><<<grid, T, smem, s>>>(nullptr, rm, rs, dst, c.ntt, (uint32_t)rows);
   else
-    k_ntt_fwd<LOGN, SRC_U32><<<grid, T, smem, s>>>(src, rm, rs, dst, c.ntt, c.p.L, rows);
+    k_ntt_fwd<LOGN, SRC_U32><<<grid, T, smem, s>>>(src, rm, rs, dst, c.ntt, (uint32_t)rows);
   return cudaGetLastError();
 }
 
@@ -520,13 +577,14 @@ cudaError_t inv_launch(const ParamCtx &c, const uint32_t *src, const RowMap &rm,
   const int T = (1 << LOGN) / 16;
   const size_t smem = ((1u << LOGN) + (1u << LOGN) / 16) * sizeof(uint32_t);
   const unsigned grid = (unsigned)(rows < kMaxGrid ? rows : kMaxGrid);
-  k_ntt_inv<LOGN><<<grid, T, smem, s>>>(src, rm, dst, c.ntt, c.p.L, rows);
+  k_ntt_inv<LOGN><<<grid, T, smem, s>>>(src, rm, dst, c.ntt, (uint32_t)rows);
   return cudaGetLastError();
 }
 
 cudaError_t fwd_any(const ParamCtx &c, const uint32_t *src, const RowMap &rm, const RawSrc &rs, uint32_t *dst,
                     uint64_t rows, cudaStream_t s, bool raw) {
   if (rows == 0) return cudaSuccess;
+  if (rows > kMaxRows) return cudaErrorInvalidValue;
   switch (c.logn) {
     case 11: return fwd_launch<11>(c, src, rm, rs, dst, rows, s, raw);
     case 12: return fwd_launch<12>(c, src, rm, rs, dst, rows, s, raw);
@@ -539,14 +597,14 @@ cudaError_t fwd_any(const ParamCtx &c, const uint32_t *src, const RowMap &rm, co
 
 cudaError_t launch_ntt_fwd(const ParamCtx &c, const uint32_t *src, uint32_t *dst, uint64_t rows, cudaStream_t s) {
   const RawSrc rs = {};
-  const RowMap rm = {0, rows ? rows : 1, 0, 1};
+  const RowMap rm(0, rows ? rows : 1, 0, 1, c.p.L);
   return fwd_any(c, src, rm, rs, dst, rows, s, false);
 }
 
 cudaError_t launch_ntt_fwd_rows(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
                                 uint32_t *dst, uint64_t rows, cudaStream_t s) {
   const RawSrc rs = {};
-  const RowMap rm = {off, G, S, 1};
+  const RowMap rm(off, G, S, 1, c.p.L);
   return fwd_any(c, src, rm, rs, dst, rows, s, false);
 }
 
@@ -562,7 +620,7 @@ cudaError_t launch_ntt_fwd_raw(const ParamCtx &c, const uint8_t *raw, int col_ma
     rs.c0 = first;
   else
     rs.poly0 = first;
-  const RowMap rm = {0, 1, 1, 1};
+  const RowMap rm(0, 1, 1, 1, c.p.L);
   return fwd_any(c, nullptr, rm, rs, dst, npolys * c.p.L, s, true);
 }
 
@@ -618,7 +676,8 @@ cudaError_t launch_ntt_inv_switch(const ParamCtx &c, const uint32_t *src, uint32
 
 cudaError_t launch_ntt_inv(const ParamCtx &c, const uint32_t *src, uint32_t *dst, uint64_t rows, cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
-  const RowMap rm = {0, rows, 0, 1};
+  if (rows > kMaxRows) return cudaErrorInvalidValue;
+  const RowMap rm(0, rows, 0, 1, c.p.L);
   switch (c.logn) {
     case 11: return inv_launch<11>(c, src, rm, dst, rows, s);
     case 12: return inv_launch<12>(c, src, rm, dst, rows, s);
@@ -630,7 +689,8 @@ cudaError_t launch_ntt_inv(const ParamCtx &c, const uint32_t *src, uint32_t *dst
 cudaError_t launch_ntt_inv_rows(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
                                 uint64_t T, uint32_t *dst, uint64_t rows, cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
-  const RowMap rm = {off, G, S, T};
+  if (rows > kMaxRows) return cudaErrorInvalidValue;
+  const RowMap rm(off, G, S, T, c.p.L);
   switch (c.logn) {
     case 11: return inv_launch<11>(c, src, rm, dst, rows, s);
     case 12: return inv_launch<12>(c, src, rm, dst, rows, s);
@@ -642,7 +702,7 @@ cudaError_t launch_ntt_inv_rows(const ParamCtx &c, const uint32_t *src, uint64_t
 cudaError_t launch_ntt_fwd_rows_t(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
                                   uint64_t T, uint32_t *dst, uint64_t rows, cudaStream_t s) {
   const RawSrc rs = {};
-  const RowMap rm = {off, G, S, T};
+  const RowMap rm(off, G, S, T, c.p.L);
   return fwd_any(c, src, rm, rs, dst, rows, s, false);
 }
 

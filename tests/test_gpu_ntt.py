@@ -51,3 +51,28 @@ def test_ntt_zero_count_is_ok():
     p = g.pir_make_params(4096, 16, 1, 1, 2)
     d = empty_u32(4)
     g.ntt_fwd(p, d, count=0)
+
+
+@pytest.mark.parametrize("n,L,count", [(2048, 3, 5), (4096, 2, 3), (8192, 1, 2), (8192, 4, 7)])
+def test_rows_on_16_byte_boundaries(n, L, count):
+    """Buffers 16 but not 32 bytes aligned give the same words as aligned ones."""
+    import torch
+    p = g.pir_make_params(n, 16, 1, 1, L)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n + count)
+    a = torch.empty(count, L, n, dtype=torch.int32, device="cuda")
+    for j, q in enumerate(p.qs):
+        a[:, j] = torch.randint(0, q, (count, n), generator=gen, dtype=torch.int32, device="cuda")
+    b = torch.empty(a.numel() + 4, dtype=torch.int32, device="cuda")[4:]
+    b.copy_(a.reshape(-1))
+    x = a.clone()
+    out = [torch.empty(count * n + 4, dtype=torch.int32, device="cuda")[k:k + count * n] for k in (0, 4)]
+    g.ntt_fwd(p, a)
+    g.ntt_fwd(p, b)
+    assert torch.equal(a.reshape(-1), b)
+    g.ntt_inv_modswitch(p, a, out[0])
+    g.ntt_inv_modswitch(p, b, out[1])
+    assert torch.equal(out[0], out[1])
+    g.ntt_inv(p, a)
+    g.ntt_inv(p, b)
+    assert torch.equal(a, x) and torch.equal(a.reshape(-1), b)
