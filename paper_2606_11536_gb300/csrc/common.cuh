@@ -79,12 +79,24 @@ pir_status_t get_param_ctx(const pir_params_t *p, const ParamCtx **out);  // cac
 // [B][count][2][L][n] in NTT form from packed [B][2][L][n] (coefficient form) and
 // reports its kernel launches; expander_fits checks ring and depth against a DB.
 struct pir_expander_impl;
-// Gadget digits (App. D.3): for every polynomial [L][n] (coefficient form, canonical)
-// of coef [polys][L][n], dig [polys][ell][n] holds the w-bit digits of the CRT lift of
-// each coefficient, w = gadget_bits(p, ell) = ceil(ceil(log2 q) / ell).
+// Gadget (App. D.3): ell digits of w = gadget_bits(p, ell) = ceil(ceil(log2 q) / ell) bits of
+// the CRT lift of a coefficient; the lift's Garner inverses gc[k][i] = q_i^-1 mod q_k (i < k).
+struct GadgetConst {
+  uint32_t gc[PIR_MAX_L][PIR_MAX_L], gc_sh[PIR_MAX_L][PIR_MAX_L];
+};
 uint32_t gadget_bits(const pir_params_t &p, uint32_t ell);
-cudaError_t launch_gadget_digits(const ParamCtx &c, const uint32_t *coef, uint64_t polys, uint32_t ell,
-                                 uint32_t *dig, cudaStream_t s);
+GadgetConst gadget_const(const pir_params_t &p);
+// gadget.cu: one level of expansion (2^lev ciphertexts per query, cur [queries << lev][2][L][n]
+// to out [queries][ostride][2][L][n], the first olimit of every query's 2^(lev+1)) and of folding
+// (2^(plog+1) to 2^plog ciphertexts per query), in NTT form; dig (ell n words per input
+// polynomial) and dhat (L times that) are scratch.  Three launches each.
+cudaError_t launch_expand_level(const ParamCtx &c, const GadgetConst &g, const uint32_t *cur, const uint32_t *key,
+                                const uint32_t *mon, const uint32_t *mon_sh, const uint32_t *perm, uint32_t queries,
+                                uint32_t lev, uint32_t ell, uint32_t ostride, uint32_t olimit, uint32_t *dig,
+                                uint32_t *dhat, uint32_t *out, cudaStream_t s);
+cudaError_t launch_fold_level(const ParamCtx &c, const GadgetConst &g, const uint32_t *cur, const uint32_t *rgsw,
+                              uint64_t query_words, uint32_t queries, uint32_t plog, uint32_t ell, uint32_t *dig,
+                              uint32_t *dhat, uint32_t *out, cudaStream_t s);
 bool expander_view(pir_expander_t h, const pir_expander_impl **out);
 bool expander_fits(const pir_expander_impl *ex, const pir_params_t &p);
 pir_status_t expand_device(const pir_expander_impl *ex, const uint32_t *packed, uint32_t B, uint32_t count,
@@ -120,10 +132,7 @@ cudaError_t launch_ntt_fwd(const ParamCtx &c, const uint32_t *src, uint32_t *dst
 cudaError_t launch_ntt_fwd_rows(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
                                 uint32_t *dst, uint64_t rows, cudaStream_t s);
 cudaError_t launch_ntt_inv(const ParamCtx &c, const uint32_t *src, uint32_t *dst, uint64_t rows, cudaStream_t s);
-// Row-mapped variants: local row r (prime r % L) reads source row
-// off + (r / G) * S + (r % G) * T.
-cudaError_t launch_ntt_inv_rows(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
-                                uint64_t T, uint32_t *dst, uint64_t rows, cudaStream_t s);
+// Forward NTT where local row r (prime r % L) reads source row off + (r / G) * S + (r % G) * T.
 cudaError_t launch_ntt_fwd_rows_t(const ParamCtx &c, const uint32_t *src, uint64_t off, uint64_t G, uint64_t S,
                                   uint64_t T, uint32_t *dst, uint64_t rows, cudaStream_t s);
 // Inverse NTT of `count` RNS polynomials src [count][L][n] with modulus switching to
@@ -279,13 +288,17 @@ __device__ __forceinline__ void mac_wide(uint64_t &acc, uint32_t a, uint32_t b) 
   asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
 
-// Full reduction of a 64-bit value mod q (q < 2^30): Barrett with mu = floor(2^64/q).
+// Full reduction of a 64-bit value mod q (q < 2^30), mu = floor(2^64 / q): x = xh 2^32 + xl, where
+// mu >> 32 = floor(2^32 / q) is the Shoup companion of 1, and that of c = 2^32 mod q =
+// 2^32 - (mu >> 32) q is the low half of mu.  Both products come out in [0, 2q).  32-bit
+// products only: the 64-bit high product and 64-bit compares it replaces took about twice
+// the instructions.
 __device__ __forceinline__ uint32_t reduce64(uint64_t x, uint32_t q, uint64_t mu) {
-  uint64_t qt = __umul64hi(x, mu);
-  uint64_t r = x - qt * q;  // in [0, 2q) (Barrett's error is at most one q here)
-  if (r >= q) r -= q;
-  if (r >= q) r -= q;
-  return (uint32_t)r;
+  const uint32_t mh = (uint32_t)(mu >> 32), ml = (uint32_t)mu, c = 0u - mh * q;
+  const uint32_t xh = (uint32_t)(x >> 32), xl = (uint32_t)x;
+  uint32_t r = shoup_mul(xh, c, ml, q) + (xl - __umulhi(xl, mh) * q);  // [0, 4q)
+  r = min(r, r - 2 * q);
+  return min(r, r - q);
 }
 
 }  // namespace gbpir
