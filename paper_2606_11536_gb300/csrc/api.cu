@@ -234,9 +234,11 @@ struct QueryCopy {
   size_t bytes;
   uint32_t rows;
 };
-QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, bool tight) {
+QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t D2, bool tight) {
   const size_t b = layout_qs_bytes(layout, nslots, Kc, layout_rows(layout, M));
-  if (!gemm_uses_digits(layout, tile, M, Kc)) return {b, 0};
+  if (!gemm_uses_digits(layout, tile, M, D2, Kc)) return {b, 0};
+  // fewer than 128 plain rows: digits (of 64 rows at least) take more than the tiles' copy
+  if (tight && layout == PIR_LAYOUT_PLAIN && tile == 0 && Kc < 128) return {b, 0};
   const uint32_t rows = gemm_digit_rows(nslots, Kc, round4(M), tight);
   const size_t d = gemm_digit_query_bytes(nslots, rows, round4(M));
   return {d > b ? d : b, rows};
@@ -455,7 +457,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   const size_t qhat_bytes = qhat_ready ? 0 : (size_t)B * Kc * 2 * L * n * 4;
   // (the stall test hook belongs to the TMA scan)
   const uint32_t qtile = stall ? 7 : o.tile;
-  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, false);
+  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, D2, false);
   const size_t out_bytes = nslots * M * D2 * 4;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   // Batch 1 on the TMA scan: the forward NTT writes the slot layout itself (pairs of
@@ -475,7 +477,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   cudaError_t ae = scratch.alloc(other_bytes + up(qc.bytes));
   if (ae == cudaErrorMemoryAllocation && qc.rows) {
     cudaGetLastError();
-    qc = query_copy(db->layout, qtile, nslots, Kc, M, true);
+    qc = query_copy(db->layout, qtile, nslots, Kc, M, D2, true);
     ae = scratch.alloc(other_bytes + up(qc.bytes));
   }
   CK(ae);
@@ -685,14 +687,14 @@ pir_status_t session_open(pir_db *db, uint32_t B, uint32_t kc_max, cudaStream_t 
   ses->o = o;
   ses->failed = PIR_OK;
   ses->qhat_bytes = (size_t)B * kc_max * ct * 4;
-  QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, false);
+  QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, p.D2, false);
   ses->stage_bytes = up(ses->qhat_bytes);
   const size_t out_bytes = nslots * M * p.D2 * 4;
   void *mem = nullptr;
   cudaError_t e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
   if (e == cudaErrorMemoryAllocation && qc.rows) {
     cudaGetLastError();
-    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, true);
+    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, p.D2, true);
     e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
   }
   ses->qs_bytes = qc.bytes;

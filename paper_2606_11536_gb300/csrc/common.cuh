@@ -196,7 +196,8 @@ cudaError_t launch_gemm_digit(const ParamCtx &c, int layout, const void *db, uin
 // residue where the other tiles' query copy takes 4.
 uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight);
 // Whether a layout's tile choice for chunks of Kc rows is the digit GEMM.
-bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t Kc);
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc);
+bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc);  // gemm_plain.cu: tile 0's choice
 
 // scan_tma.cu: the same contract for M <= 8 rows and D2 <= 512 (D2 % 4 == 0), as a
 // TMA-staged stream; stall_test makes its consumers wait on a barrier that never
@@ -208,6 +209,10 @@ bool scan_tma_supports(uint32_t M, uint32_t D2);
 cudaError_t launch_scan_tma(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
                             uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc, int stall_test,
                             int out_poly, const uint32_t *acc_src, cudaStream_t s);
+// The same product with the rows read straight from global memory, any M.
+cudaError_t launch_scan_direct(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
+                               uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
+                               int out_poly, const uint32_t *acc_src, cudaStream_t s);
 
 // gemm_limb.cu: the same contract on the limb layouts (db [s][4][D2][D1] u8,
 // ql [s][4][Mp][Kc] u8), exact through u8 x u8 -> s32 tensor-pipe products.

@@ -620,18 +620,14 @@ uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight) 
   return r < 64 ? 64 : r > kDigitMaxRows ? kDigitMaxRows : r;
 }
 
-bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t Kc) {
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc) {
   if (layout == PIR_LAYOUT_TENSOR) return false;
   if (tile == (layout == PIR_LAYOUT_PLAIN ? kDigitTile : kLimbDigitTile)) return true;
   if (tile != 0 || !gemm_digit_available()) return false;
   // INT8 mma.sync at its peak is 1.3 to 7 times slower at every size measured (32 to 512 rows
   // and columns, 1 to 32 queries).
   if (layout == PIR_LAYOUT_LIMB) return true;
-  // One query streams the DB at HBM speed on the CUDA cores already.  From 128 rows on the
-  // digit GEMM wins at every width (1.2x at 512 columns and batch 4, up to 4x); at 64 rows
-  // it still wins at 32 columns (1.5-3x) but loses at 256 (0.78-1.06x), where its
-  // epilogue outweighs the products.
-  return M >= 3 && Kc >= 128;
+  return gemm_plain_digits(M, D2, Kc);
 }
 
 bool gemm_digit_available() { return tensor_maps_available(); }

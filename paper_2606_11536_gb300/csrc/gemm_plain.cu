@@ -300,8 +300,54 @@ cudaError_t gemm_launch(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint
 
 }  // namespace
 
+namespace {
+constexpr uint32_t kScanCols = 512;
+constexpr float kMargin = 0.85f;
+
+// What an answer takes by each path, in us per 4096 slots: fitted to 880 shapes (D1 16 to 256,
+// D2 16 to 512, 2 to 64 queries; 6 to 14% rms).  A path other than the tiles is taken where
+// its estimate is 15% below theirs: on average 2% off the best path, where digits from 128 rows
+// on and the tiles below were 41% (up to 4.6 times) off.  Where digits pay: 127 x 16, 12
+// queries, 640 us by the tile, 139 by digits; 64 x 64, 8 queries, 206 and 116; but 64 x 512, 4
+// queries, 270 and 348.  Where the direct scan does: 16 x 16, 16 queries, 128 and 80; 64 x 16, 4
+// queries, 126 and 53; but 64 x 128, 8 queries, 219 and 211 (178 by digits).
+struct Costs {
+  float digit, core, direct;
+};
+Costs costs(uint32_t M, uint32_t D2, uint32_t Kc) {
+  auto up = [](uint32_t x, uint32_t m) { return (float)((x + m - 1) / m * m); };
+  const float K = (float)Kc, cells = (float)M * D2;
+  Costs t;
+  // digits: unit epilogues over columns packed to 32, 64 or 128, K padded to 64 rows
+  const uint32_t least = M > 32 ? 64 : 32;
+  const float cols = D2 <= least ? (float)least : D2 <= 64 ? 64.f : up(D2, 128);
+  t.digit = 43.2f + (0.0736f + (M > 32 ? 0.0393f : 0.0531f) * up(M, 8)) * cols + 0.0172f * up(Kc, 64) * M;
+  // the CUDA-core GEMM tiles: products of whole tiles
+  const uint32_t tm = M <= 8 ? 8 : M <= 16 ? 16 : M <= 32 ? 32 : 64;
+  t.core = 39.1f + 0.0211f * cells + 0.0181f * K * M +
+           (tm == 8 ? 5.9e-4f : 5.0e-4f) * (K < 16 ? 16 : K) * up(D2, tm == 64 ? 128 : 256) * up(M, tm);
+  // the direct scan: products of lanes over strips of 128 columns, padded to a power of two
+  uint32_t lanes = D2 / 128 * 128, rest = D2 % 128, p2 = 4;
+  if (rest) {
+    while (p2 < rest) p2 *= 2;
+    lanes += p2;
+  }
+  t.direct = 38.3f + 0.01625f * cells + 9.6e-4f * up(M, M > 4 ? 8 : 4) * lanes * K + 0.0221f * K * M;
+  return t;
+}
+}  // namespace
+
+// One query streams the DB at HBM speed on the CUDA cores already.  From 128 rows on the digit
+// GEMM wins at every width (1.2x at 512 columns and batch 4, up to 4x).
+bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc) {
+  if (M < 3) return false;
+  if (Kc >= 128) return true;
+  const Costs t = costs(M, D2, Kc);
+  return (t.digit < t.direct || D2 > kScanCols) && (M <= 4 || t.digit < kMargin * t.core);
+}
+
 // Tile ids: 1 = GEMV MB=2, 2 = GEMV MB=4, 3 = GEMV MB=8, 4 = GEMM 16x256, 5 = GEMM 32x256,
-// 6 = GEMM 64x128, 7 = TMA-staged scan (M <= 8, D2 <= 512; scan_tma.cu), 8 = GEMM 8x256
+// 6 = GEMM 64x128, 7 = scan (M <= 8, D2 <= 512; staged by TMA or direct, scan_tma.cu), 8 = GEMM 8x256
 // (one query row per thread, for a few queries).  Where the digit GEMM does not apply, 0
 // picks the TMA scan up to 4 rows, the 8-row GEMM up to 8, else a GEMM tile by M.
 // 9 = the tensor-core GEMM over in-kernel digits (gemm_digit.cu), which takes another
@@ -324,9 +370,11 @@ cudaError_t launch_gemm_plain(const ParamCtx &c, const uint32_t *db, uint32_t D1
                               uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
                               uint32_t tile, int stall_test, cudaStream_t s) {
   if (tile == 0) {
-    // measured on GB300: the TMA scan wins up to 4 query rows; with 6-8 rows its
-    // accumulators cap it at one or two CTAs per SM and the GEMV-shaped kernel wins
-    // (5-8 rows: the 8-row GEMM tile measured 15-17% ahead of the GEMV)
+    // the scans up to 4 query rows; from 5 on the direct scan against the GEMM tile that holds
+    // the rows (5-8 rows: the 8-row GEMM tile measured 15-17% ahead of the GEMV)
+    const Costs t = costs(M, D2, Kc);
+    if (D2 <= kScanCols && M > 4 && t.direct < kMargin * t.core)
+      return launch_scan_direct(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, 0, nullptr, s);
     if (M <= 4 && scan_tma_supports(M, D2)) tile = 7;
     else if (M <= 2) tile = 1;
     else if (M <= 4) tile = 2;

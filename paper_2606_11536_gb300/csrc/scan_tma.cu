@@ -1,4 +1,4 @@
-// scan_tma.cu -- the batch-1..4 first-dimension scan as a TMA-staged stream over
+// scan_tma.cu -- the first-dimension scan for a few queries: as a TMA-staged stream over
 // the resident NTT-form DB (the memory-bound GEMV of Sec. 5 / the (#RNS*N)-parallel
 // modular GEMMs of Sec. 4.2 with 2B <= 8 query rows).
 //
@@ -261,6 +261,122 @@ __global__ void __launch_bounds__(kThreads, ScanShape<MB, T>::kMinBlocks) k_scan
   }
 }
 
+// The direct scan: one warp per slot and strip of 128 columns, DB rows read straight from
+// global memory; lane = (row phase, quad of columns).  A block's eight neighbouring slots
+// meet in shared memory so that the response layout is written in whole 32-byte sectors.
+// More than eight query rows take a pass per eight, the slot's DB rows then from L2.
+// The staged stream costs about 3.5 us per slot and CTA whatever a slot's size (waits, folds and
+// shuffles of eight warps), and a row narrower than its eight warps' quads leaves warps without
+// work.  One query, n = 2^12, L = 2, staged -> direct: 16 x 16 49 -> 12 us, 64 x 32 94 -> 26, 256 x 64
+// 287 -> 123 (4.4 TB/s), 1024 x 16 534 -> 129.
+constexpr int kDirectWarps = 8, kDirectUnroll = 4;
+constexpr uint32_t kDirectCols = 128;
+
+template <int MB>
+__global__ void __launch_bounds__(kDirectWarps * 32) k_scan_direct(ScanArgs a, ModConst mc) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  uint32_t *tile = reinterpret_cast<uint32_t *>(smem);  // [M][cols][kDirectWarps + 1]
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t s0 = blockIdx.x * kDirectWarps, s = s0 + warp;
+  const uint32_t c0 = blockIdx.y * kDirectCols, cols = min(kDirectCols, a.D2 - c0), nq = cols >> 2;
+  uint32_t QW = 1;
+  while (QW < nq) QW <<= 1;
+  const uint32_t PH = 32 / QW, ql = lane & (QW - 1), phs = lane / QW;
+  const bool qv = ql < nq;
+  const uint32_t j = s >> a.logn;
+  uint32_t q = mc.q[0];
+  uint64_t mu = mc.mu[0], k63 = mc.k63[0];
+#pragma unroll
+  for (uint32_t i = 1; i < PIR_MAX_L; ++i)
+    if (i == j) q = mc.q[i], mu = mc.mu[i], k63 = mc.k63[i];
+  const uint32_t *db = a.db + ((uint64_t)s * a.D1 + a.i0) * a.D2 + c0 + 4 * (qv ? ql : 0);
+  const uint32_t m0 = blockIdx.z * MB, M = min(a.M - m0, (uint32_t)MB);  // this block's query rows
+  const uint32_t *qs = a.qs + (uint64_t)s * a.Kc * a.Mp + m0;
+  uint64_t acc[MB][4] = {};
+  bool full = false;  // every second group of kDirectUnroll products
+  for (uint32_t r0 = phs; r0 < a.Kc; r0 += kDirectUnroll * PH) {
+    uint32_t qrow[kDirectUnroll][MB];
+    uint4 d[kDirectUnroll];
+#pragma unroll
+    for (int u = 0; u < kDirectUnroll; ++u) {
+      const uint32_t r = r0 + u * PH, rc = r < a.Kc ? r : a.Kc - 1;
+      d[u] = __ldg(reinterpret_cast<const uint4 *>(db + (uint64_t)rc * a.D2));
+      if constexpr (MB == 2) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(qs + rc * a.Mp));
+        qrow[u][0] = v.x, qrow[u][1] = v.y;
+      } else {
+#pragma unroll
+        for (int m = 0; m < MB; m += 4) {
+          const uint4 v = m < (int)M ? __ldg(reinterpret_cast<const uint4 *>(qs + rc * a.Mp + m)) : make_uint4(0, 0, 0, 0);
+          qrow[u][m] = v.x, qrow[u][m + 1] = v.y, qrow[u][m + 2] = v.z, qrow[u][m + 3] = v.w;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kDirectUnroll; ++u) {
+      const bool rv = r0 + u * PH < a.Kc;
+#pragma unroll
+      for (int m = 0; m < MB; ++m) {
+        const uint32_t x = rv ? qrow[u][m] : 0;
+        mac_wide(acc[m][0], x, d[u].x);
+        mac_wide(acc[m][1], x, d[u].y);
+        mac_wide(acc[m][2], x, d[u].z);
+        mac_wide(acc[m][3], x, d[u].w);
+      }
+    }
+    if (full) {
+#pragma unroll
+      for (int m = 0; m < MB; ++m)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[m][e] = fold63(acc[m][e], k63);
+    }
+    full = !full;
+  }
+#pragma unroll
+  for (int m = 0; m < MB; ++m) {
+    uint32_t r[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      uint32_t v = reduce64(acc[m][e], q, mu);
+      for (uint32_t off = QW; off < 32; off <<= 1) {
+        v += __shfl_xor_sync(0xffffffffu, v, off);
+        v = min(v, v - q);
+      }
+      r[e] = v;
+    }
+    if (phs == 0 && qv && (uint32_t)m < M) {
+      const uint64_t at = ((uint64_t)s * a.M + m0 + m) * a.D2 + c0 + 4 * ql;
+      if (a.acc_src || a.acc_in) {  // earlier K-chunks, slot-major
+        const uint4 prev = *reinterpret_cast<const uint4 *>((a.acc_src ? a.acc_src : a.out) + at);
+        r[0] += prev.x, r[1] += prev.y, r[2] += prev.z, r[3] += prev.w;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) r[e] = min(r[e], r[e] - q);
+      }
+      if (a.out_poly) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) tile[(m * cols + 4 * ql + e) * (kDirectWarps + 1) + warp] = r[e];
+      } else {
+        *reinterpret_cast<uint4 *>(a.out + at) = make_uint4(r[0], r[1], r[2], r[3]);
+      }
+    }
+  }
+  if (!a.out_poly) return;
+  __syncthreads();
+  const uint32_t k = threadIdx.x % kDirectWarps;
+  for (uint32_t m = 0; m < M; ++m)
+    for (uint32_t c = threadIdx.x / kDirectWarps; c < cols; c += 32)
+      a.out[(((uint64_t)(m >> 1) * a.D2 + c0 + c) * 2 + (m & 1)) * a.nslots + s0 + k] =
+          tile[(m * cols + c) * (kDirectWarps + 1) + k];
+}
+
+template <int MB>
+cudaError_t direct_launch(const ParamCtx &c, const ScanArgs &a, cudaStream_t s) {
+  const size_t smem = a.out_poly ? (size_t)a.M * kDirectCols * (kDirectWarps + 1) * 4 : 0;  // 36 KiB at most
+  const dim3 grid(a.nslots / kDirectWarps, (a.D2 + kDirectCols - 1) / kDirectCols, (a.M + MB - 1) / MB);
+  k_scan_direct<MB><<<grid, kDirectWarps * 32, smem, s>>>(a, c.mod);
+  return cudaGetLastError();
+}
+
 template <int MB, int T>
 cudaError_t scan_launch(const ParamCtx &c, const ScanArgs &a0, cudaStream_t s) {
   int dev = 0, sms = 0;
@@ -283,6 +399,40 @@ cudaError_t scan_launch(const ParamCtx &c, const ScanArgs &a0, cudaStream_t s) {
 
 }  // namespace
 
+namespace {
+// Whether the staged stream is the faster scan.  It is where a row fills its eight warps' quads
+// (one or two each) and a slot is long enough; one query: 64 x 256 112 against 123 us direct,
+// 512 x 256 654 against 797, 256 x 460 629 against 818; but 16 x 256 58 against 45, 32 x 512 135
+// against 122, 256 x 160 (by rate) and 256 x 400 847 against 672.  Two queries: 512 x 256 1060
+// against 1127, 512 x 512 3040 against 2136, 64 x 256 188 against 164.  Four: always slower.
+bool staged_wins(uint32_t M, uint32_t D2, uint32_t Kc) {
+  const uint64_t bytes = (uint64_t)Kc * D2 * 4;
+  if (D2 <= 256) return D2 >= 192 && (M <= 2 ? bytes >= (64u << 10) : M <= 4 && bytes >= (128u << 10));
+  return D2 >= 448 && M <= 2 && bytes >= (128u << 10);
+}
+}  // namespace
+
+cudaError_t launch_scan_direct(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
+                               uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
+                               int out_poly, const uint32_t *acc_src, cudaStream_t s) {
+  ScanArgs a = {};
+  a.db = db;
+  a.qs = qs;
+  a.out = out;
+  a.M = M;
+  a.Mp = Mp;
+  a.D1 = D1;
+  a.D2 = D2;
+  a.i0 = i0;
+  a.Kc = Kc;
+  a.nslots = c.p.L << c.logn;
+  a.logn = c.logn;
+  a.acc_in = acc;
+  a.out_poly = out_poly;
+  a.acc_src = acc_src;
+  return M <= 2 ? direct_launch<2>(c, a, s) : M <= 4 ? direct_launch<4>(c, a, s) : direct_launch<8>(c, a, s);
+}
+
 // The TMA scan holds M <= 8 rows and D2 <= 8 * 8 * 4 * 2 = 512 columns per lane
 // budget (T <= 2 quads per lane).
 bool scan_tma_supports(uint32_t M, uint32_t D2) { return M <= 8 && D2 % 4 == 0 && D2 <= 512; }
@@ -293,6 +443,8 @@ cudaError_t launch_scan_tma(const ParamCtx &c, const uint32_t *db, uint32_t D1, 
   // query rows are bulk-copied: Mp = 2 needs an even Kc (16-byte chunk starts)
   if (!scan_tma_supports(M, D2) || Kc == 0 || !(Mp % 4 == 0 || (Mp == 2 && M <= 2 && Kc % 2 == 0)))
     return cudaErrorInvalidValue;
+  if (!stall_test && !staged_wins(M, D2, Kc))
+    return launch_scan_direct(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, out_poly, acc_src, s);
   uint32_t *err = nullptr;
   cudaError_t e = device_error_word(&err);
   if (e != cudaSuccess) return e;
