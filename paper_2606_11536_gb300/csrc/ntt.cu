@@ -308,8 +308,10 @@ cudaError_t pair_launch(const ParamCtx &c, const uint32_t *src, uint64_t row0, u
                         uint32_t col0, uint32_t *slots, cudaStream_t s) {
   const int T = (1 << LOGN) / 8;  // two rows in parallel
   const int smem = 2 * ((1 << LOGN) + (1 << LOGN) / 16) * (int)sizeof(uint32_t);
-  cudaError_t e = cudaFuncSetAttribute(k_ntt_fwd_pair_slots<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024 &&  // above the limit a kernel has without asking
+      (e = cudaFuncSetAttribute(k_ntt_fwd_pair_slots<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    return e;
   k_ntt_fwd_pair_slots<LOGN><<<kc * c.p.L, T, smem, s>>>(src, row0, c.ntt, c.p.L, stride, col0, slots);
   return cudaGetLastError();
 }
@@ -332,8 +334,10 @@ cudaError_t switch_launch(const ParamCtx &c, const uint32_t *src, uint32_t *dst,
   constexpr int N = 1 << LOGN, PADN = N + N / 16;
   const uint32_t L = c.p.L;
   const int smem = (int)(L * PADN * sizeof(uint32_t));
-  cudaError_t e = cudaFuncSetAttribute(k_ntt_inv_switch<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024 &&  // above the limit a kernel has without asking
+      (e = cudaFuncSetAttribute(k_ntt_inv_switch<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    return e;
   for (uint64_t first = 0; first < count; first += kMaxGrid) {
     const uint64_t nb = count - first < kMaxGrid ? count - first : kMaxGrid;
     k_ntt_inv_switch<LOGN><<<(unsigned)nb, N / 8, smem, s>>>(src + first * L * N, dst + first * N, c.ntt, c.sw, L);
