@@ -346,10 +346,11 @@ struct StageTimer {
 
 // One K-chunk on the DB's GEMM path: the NTT-form chunk qhat [B][kc][2][L][n] to
 // the layout's query copy qs, then the GEMM accumulated into out [L*n][M][D2].
-// digit_rows: the digit GEMM in pieces of so many rows (query_copy).
+// digit_rows: the digit GEMM in pieces of so many rows (query_copy).  queries, when set: the
+// coefficient-form queries [B][D1][2][L][n] instead of qhat; their NTT writes the digits.
 pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint32_t Mp, uint32_t i0, uint32_t kc,
                         uint32_t digit_rows, void *qs, uint32_t *out, uint32_t tile, int stall, StageTimer &tm,
-                        cudaStream_t s) {
+                        cudaStream_t s, const uint32_t *queries = nullptr) {
   const ParamCtx &c = *db->ctx;
   const uint32_t D1 = db->p.D1, D2 = db->p.D2, M = 2 * B;
   if (digit_rows) {
@@ -357,8 +358,11 @@ pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint
     for (uint32_t k0 = 0; k0 < kc; k0 += digit_rows) {
       const uint32_t kr = kc - k0 < digit_rows ? kc - k0 : digit_rows;
       tm.begin();
-      CK(launch_query_digits(c, db->layout, qhat, B, kc, k0, kr, round4(M), qt, s));
-      tm.end(1, 1);
+      if (queries)
+        CK(launch_ntt_query_digits(c, db->layout, queries, B, D1, i0 + k0, kr, round4(M), qt, s));
+      else
+        CK(launch_query_digits(c, db->layout, qhat, B, kc, k0, kr, round4(M), qt, s));
+      tm.end(queries ? 0 : 1, 1);
       tm.begin();
       CK(launch_gemm_digit(c, db->layout, db->resident, D1, D2, qt, M, round4(M), i0 + k0, kr, out, i0 + k0 > 0, s));
       tm.end(2, 1);
@@ -370,9 +374,11 @@ pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint
     CK(launch_query_to_slots(c, qhat, B, kc, Mp, static_cast<uint32_t *>(qs), s));
   else if (db->layout == PIR_LAYOUT_LIMB)
     CK(launch_query_to_limbs(c, qhat, B, kc, Mp, static_cast<uint8_t *>(qs), s));
+  else if (queries)
+    CK(launch_ntt_query_digits(c, db->layout, queries, B, D1, i0, kc, Mp, static_cast<uint16_t *>(qs), s));
   else
     CK(launch_query_to_tensor(c, qhat, B, kc, Mp, static_cast<uint16_t *>(qs), s));
-  tm.end(1, 1);
+  tm.end(queries ? 0 : 1, 1);
   tm.begin();
   if (db->layout == PIR_LAYOUT_PLAIN)
     CK(launch_gemm_plain(c, static_cast<const uint32_t *>(db->resident), D1, D2, static_cast<const uint32_t *>(qs), M,
@@ -538,13 +544,16 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // forward NTT of ciphertexts i0 .. i0+kc-1 of every query: per query b the rows
     // (b*D1 + i0)*2L .. +kc*2L are contiguous.
     const uint64_t G = (uint64_t)kc * 2 * L, S = (uint64_t)D1 * 2 * L;
-    if (!qhat_ready) {
+    const bool digits = db->layout == PIR_LAYOUT_TENSOR || qc.rows;
+    const bool direct = !qhat_ready && digits && query_ntt_fuses(c, B, kc);
+    if (!qhat_ready && !direct) {
       tm.begin();
       CK(launch_ntt_fwd_rows(c, queries, (uint64_t)i0 * 2 * L, G, S, const_cast<uint32_t *>(qhat), (uint64_t)B * G,
                              s));
       tm.end(0, 1);
     }
-    const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, qc.rows, qs, out, o.tile, stall, tm, s);
+    const pir_status_t st = chunk_gemm(db, qhat, B, Mp, i0, kc, qc.rows, qs, out, o.tile, stall, tm, s,
+                                       direct ? queries : nullptr);
     if (st != PIR_OK) return st;
   }
   tm.begin();

@@ -199,6 +199,13 @@ uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight);
 bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc);
 bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc);  // gemm_plain.cu: tile 0's choice
 
+// query_ntt.cu: ciphertexts i0 .. i0 + Kc - 1 of every query (queries [B][D1][2][L][n], coefficient
+// form) to the digits that launch_query_digits (plain, limb) or launch_query_to_tensor make of
+// their transforms, in one launch; and whether there are rows enough for it.
+bool query_ntt_fuses(const ParamCtx &c, uint32_t B, uint32_t Kc);
+cudaError_t launch_ntt_query_digits(const ParamCtx &c, int layout, const uint32_t *queries, uint32_t B, uint32_t D1,
+                                    uint32_t i0, uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s);
+
 // scan_tma.cu: the same contract for M <= 8 rows and D2 <= 512 (D2 % 4 == 0), as a
 // TMA-staged stream; stall_test makes its consumers wait on a barrier that never
 // completes (exercises the bounded-wait error path).
