@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(TcArgs a, ModConst mc) 
   const uint32_t tfull0 = saddr(bars + 2 * kMaxStages), tempty0 = saddr(bars + 2 * kMaxStages + 2);
   const uint32_t done = saddr(bars + 2 * kMaxStages + 4);
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kMaxStages + 5);
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t R = 4 * a.D2, U = a.D1 / 16, Uc = a.Kc / 16;
   const uint32_t nst = Uc / a.KS16, Ntot = 4 * a.Mp;
   const uint32_t db_stage = a.KS16 * a.T * kBlockBytes;
@@ -304,27 +304,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(TcArgs a, ModConst mc) 
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      uint32_t it = 0, k = 0;
-      bool ok = true;
-      for (uint32_t gi = cl0; ok && gi < ngroups; gi += ncl, ++k) {
-        const Unit w = unit_of(a, gi * C + rank);
-        const uint32_t buf = k % a.nbuf, use = k / a.nbuf;
-        if (!wait_bounded(tempty0 + 8 * buf, (use & 1) ^ 1)) {  // the epilogue has drained this buffer
-          atomicExch(a.err, 1u);
-          break;
-        }
+    // the whole warp runs the loop, so that its state stays warp-uniform; one lane issues.
+    // (One lane running the loop alone took 1.4 times as long per MMA in the pair form.)
+    tcgen::Ring r;
+    uint32_t k = 0;
+    bool ok = true, ready = false;
+    auto wait = [&](uint32_t bar, uint32_t parity) { ok = __all_sync(0xffffffffu, wait_bounded(bar, parity)) && ok; };
+    for (uint32_t gi = cl0; ok && gi < ngroups; gi += ncl, ++k) {
+      const Unit w = unit_of(a, gi * C + rank);
+      const uint32_t buf = k % a.nbuf, use = k / a.nbuf;
+      wait(tempty0 + 8 * buf, (use & 1) ^ 1);  // the epilogue has drained this buffer
+      if (!ok) break;
+      const uint32_t idesc = instr_desc(128, w.Nt), dcol = tmem + buf * a.buf_cols;
+      for (uint32_t st = 0; st < nst; ++st) {
+        if (!ready) wait(full0 + 8 * r.slot, r.phase);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t idesc = instr_desc(128, w.Nt), dcol = tmem + buf * a.buf_cols;
-        for (uint32_t st = 0; st < nst; ++st, ++it) {
-          const uint32_t slot = it % a.S;
-          if (!wait_bounded(full0 + 8 * slot, (it / a.S) & 1)) {
-            atomicExch(a.err, 1u);
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t base = saddr(smem + slot * a.stage_bytes);
+        const uint32_t slot = r.slot, base = saddr(smem + slot * a.stage_bytes);
+        // the next stage's barrier is looked up before these MMAs and its answer read after them:
+        // a wait costs about 100 cycles even where it is over
+        r.next(a.S);
+        const bool next = tcgen::mbar_test(full0 + 8 * r.slot, r.phase);
+        if (tcgen::elect_one()) {
           for (uint32_t v = 0; v < a.KS16; ++v) {
             const uint64_t bdesc = smem_desc(base + db_stage + v * w.Nt * 32);
             for (uint32_t t = 0; t < a.T; ++t) {
@@ -337,16 +338,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(TcArgs a, ModConst mc) 
             mma_commit(empty0 + 8 * slot);
           else
             mma_commit_multicast(empty0 + 8 * slot, all_ctas);
+          if (st + 1 == nst) mma_commit(tfull0 + 8 * buf);  // this unit's accumulators are complete
         }
-        mma_commit(tfull0 + 8 * buf);  // this unit's accumulators are complete
+        __syncwarp();
+        ready = __all_sync(0xffffffffu, next);
       }
-      // on every path: no MMA may still be running when the tensor memory is freed
-      mma_commit(done);
-      if (!wait_bounded(done, 0)) atomicExch(a.err, 1u);
     }
+    if (!ok && lane == 0) atomicExch(a.err, 1u);
+    // on every path: no MMA may still be running when the tensor memory is freed
+    if (tcgen::elect_one()) mma_commit(done);
     __syncwarp();
+    if (!__all_sync(0xffffffffu, wait_bounded(done, 0)) && lane == 0) atomicExch(a.err, 1u);
   } else {
-    // ---------------- epilogue: warps 0..7 ----------------
+    // ---------------- epilogue ----------------
     const uint32_t quarter = warp & 3, b = lane & 3;
     const uint32_t row = 32 * quarter + lane;  // accumulator lane: column c_local = row / 4, DB digit b
     const bool hi2 = (b & 2) != 0, hi1 = (b & 1) != 0;
@@ -450,6 +454,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(TcArgs a, ModConst mc) 
 //               (2 x kEpiWarps arrivals, the odd CTA's remote)
 // Every wait is bounded; the end is a cluster barrier, after which both CTAs
 // release the pair's tensor memory.
+//
+// Bound by HBM: 512 x 256, 32 queries, n = 2^12, L = 2 reads 9.7 GB in 1.58 ms (6.1 TB/s).  It took
+// 2.15 ms with one lane running the MMA loop (divergent: every step of it on the general
+// path, each MMA later) and a cluster-scope release on the epilogue's arrive, which waited for the
+// warp's stores before the buffer could be filled again.
 
 __device__ __forceinline__ void mma_bf16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                               uint32_t accumulate) {
@@ -513,7 +522,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t tfull0 = saddr(bars + 3 * kMaxStages2), tempty0 = saddr(bars + 3 * kMaxStages2 + 2);
   const uint32_t done = saddr(bars + 3 * kMaxStages2 + 4);
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 3 * kMaxStages2 + 5);
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank(), cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
   const uint32_t R = 4 * a.D2, U = a.D1 / 16, Uc = a.Kc / 16;
   const uint32_t nst = Uc / a.KS16, Ntot = 4 * a.Mp;
@@ -610,47 +619,58 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
           mbar_arrive_cluster(pfull0 + 8 * (it % a.S), 0);
         }
-    } else if (lane == 0 && rank == 0) {
-      uint32_t it = 0, k = 0;
-      bool ok = true;
+    } else if (rank == 0) {
+      // the whole warp runs the loop, so that its state stays warp-uniform; one lane issues
+      tcgen::Ring r;
+      uint32_t k = 0;
+      bool ok = true, ready = false;
+      auto wait = [&](uint32_t bar, uint32_t parity) {
+        ok = __all_sync(0xffffffffu, wait_bounded(bar, parity)) && ok;
+      };
       for (uint32_t u = cluster; ok && u < a.nunits; u += nclusters, ++k) {
         const Unit w = unit_of_pair(a, u, 0);
         const uint32_t buf = k % a.nbuf, use = k / a.nbuf, half = w.Nt / 2;
-        if (!wait_bounded(tempty0 + 8 * buf, (use & 1) ^ 1)) {  // both epilogues have drained this buffer
-          atomicExch(a.err, 1u);
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        wait(tempty0 + 8 * buf, (use & 1) ^ 1);  // both epilogues have drained this buffer
+        if (!ok) break;
         const uint32_t idesc = instr_desc(256, w.Nt), dcol = tmem + buf * a.buf_cols;
-        for (uint32_t st = 0; st < nst; ++st, ++it) {
-          const uint32_t slot = it % a.S, ph = (it / a.S) & 1;
-          if (!wait_bounded(full0 + 8 * slot, ph) || (!TMA && !wait_bounded(pfull0 + 8 * slot, ph))) {
-            atomicExch(a.err, 1u);
-            ok = false;
-            break;
-          }
+        for (uint32_t st = 0; st < nst; ++st) {
+          if (!ready) wait(full0 + 8 * r.slot, r.phase);
+          if (!TMA && ok) wait(pfull0 + 8 * r.slot, r.phase);
+          if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t base = saddr(smem + slot * a.stage_bytes);
-          for (uint32_t v = 0; v < a.KS16; ++v) {
-            const uint64_t adesc = smem_desc(base + v * kBlockBytes);
-            const uint64_t bdesc = smem_desc(base + db_stage + v * half * 32);
-            mma_bf16_pair(dcol, adesc, bdesc, idesc, (st | v) != 0);
+          const uint32_t slot = r.slot, base = saddr(smem + slot * a.stage_bytes);
+          const uint64_t adesc = smem_desc(base), bdesc = smem_desc(base + db_stage);
+          // the next stage's barrier is looked up before these MMAs and its answer read after
+          // them: a wait costs about 100 cycles even where it is over
+          r.next(a.S);
+          const bool next = tcgen::mbar_test(full0 + 8 * r.slot, r.phase);
+          if (tcgen::elect_one()) {
+#pragma unroll
+            for (uint32_t v = 0; v < 4; ++v)
+              if (v < a.KS16)
+                mma_bf16_pair(dcol, adesc + v * (kBlockBytes >> 4), bdesc + v * (half * 32 >> 4), idesc, (st | v) != 0);
+            mma_commit_pair(empty0 + 8 * slot);  // both CTAs' stage is free once these MMAs have read it
+            if (st + 1 == nst) mma_commit_pair(tfull0 + 8 * buf);  // this unit's accumulators are complete
           }
-          mma_commit_pair(empty0 + 8 * slot);  // both CTAs' stage is free once these MMAs have read it
+          __syncwarp();
+          ready = __all_sync(0xffffffffu, next);
         }
-        mma_commit_pair(tfull0 + 8 * buf);  // this unit's accumulators are complete in both CTAs
       }
+      if (!ok && lane == 0) atomicExch(a.err, 1u);
       // on every path: no MMA may still be running when the tensor memory is freed
-      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
-                   : "memory");
-      if (!wait_bounded(done, 0)) atomicExch(a.err, 1u);
+      if (tcgen::elect_one())
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
+                     : "memory");
+      __syncwarp();
+      if (!__all_sync(0xffffffffu, wait_bounded(done, 0)) && lane == 0) atomicExch(a.err, 1u);
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: warps 0..7 of each CTA, on its own accumulator rows ----------------
+    // ---------------- epilogue warps of each CTA, on its own accumulator rows ----------------
     const uint32_t quarter = warp & 3, b = lane & 3;
     const uint32_t row = 32 * quarter + lane;  // accumulator lane: column c_local = row / 4, DB digit b
     const bool hi2 = (b & 2) != 0, hi1 = (b & 1) != 0;
+    const uint32_t tempty_lead = tcgen::map_to_rank(tempty0, 0);
     uint32_t k = 0;
     for (uint32_t u = cluster; u < a.nunits; u += nclusters, ++k) {
       const Unit w = unit_of_pair(a, u, rank);
@@ -708,7 +728,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty0 + 8 * buf, 0);
+      if (lane == 0) tcgen::mbar_arrive_at(tempty_lead + 8 * buf);
     }
   }
 
