@@ -270,6 +270,31 @@ struct FastDiv {
   __device__ __forceinline__ uint32_t mod(uint32_t n) const { return n - div(n) * d; }
 };
 
+// Short kernels of one chain overlap: a kernel launched by launch_chained may start while the one
+// before it in the stream drains, and waits in chain_wait, before its first global access, until
+// that one is complete and its writes are visible; it then lets its own successor start
+// (whose blocks fill the SMs only once all of this kernel's have begun).  The gap it closes is 1 to
+// 2 us a launch: smallest answer (three launches) 18.8 -> 15.5 us, 26 folding launches 432 -> 380,
+// expansion of one query by 16 108 -> 73 us, 1001 inverse rows x 3 of n = 2^13 67.6 -> 64.8.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, uint32_t block, size_t smem, cudaStream_t s, A &&...args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Shoup multiplication by a constant w < q with wsh = floor(w * 2^32 / q):
 // returns x * w mod q in [0, 2q) for any x < 2^32 (needs q < 2^31).
 __device__ __forceinline__ uint32_t shoup_mul(uint32_t x, uint32_t w, uint32_t wsh, uint32_t q) {

@@ -44,6 +44,7 @@ __global__ void k_expand_scale(uint32_t *__restrict__ x, uint32_t n, uint32_t L,
   for (uint32_t k = 1; k < PIR_MAX_L; ++k)
     if (i == k) q = E.q[k], w = E.inv2l[k], wsh = E.inv2l_sh[k];
   uint4 *row = reinterpret_cast<uint4 *>(x + (uint64_t)blockIdx.x * n);
+  chain_wait();
   for (uint32_t e = threadIdx.x; e < n / 4; e += blockDim.x) {
     uint4 v = row[e];
     v.x = shoup_mul(v.x, w, wsh, q), v.x = min(v.x, v.x - q);
@@ -151,8 +152,7 @@ pir_status_t expand_device(const pir_expander_impl *ex, const uint32_t *packed, 
     const uint32_t nb = B - b0 < Bc ? B - b0 : Bc;
     // level-0 input: NTT of the packed ciphertexts, times 2^-levels
     if (!ck(launch_ntt_fwd(c, packed + (uint64_t)b0 * ctw, cur, (uint64_t)nb * 2 * L, s))) break;
-    k_expand_scale<<<nb * 2 * L, 256, 0, s>>>(cur, n, L, ex->scale);
-    if (!ck(cudaGetLastError())) break;
+    if (!ck(launch_chained(k_expand_scale, nb * 2 * L, 256, 0, s, cur, n, L, ex->scale))) break;
     launches += 2;
     for (uint32_t lev = 0; lev < levels; ++lev) {
       const bool last = lev + 1 == levels;

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kGroups<LOGN, L> << (LOGN - 4),
   const uint32_t grp = threadIdx.x / T, tid = threadIdx.x % T;
   const bool wide = wide_ok(cur);
   const uint64_t ctw = 2ull * L * N;
+  chain_wait();
   const uint32_t *src = FOLD ? cur + (blockIdx.x >> 1) * 2 * ctw + (blockIdx.x & 1) * (L * N) : cur + blockIdx.x * ctw;
 #pragma unroll 1
   for (uint32_t j0 = 0; j0 < L; j0 += G) {
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(kMacThreads) k_gadget_mac(const MacArgs a) {
   const uint64_t mu = pick(a.mod.mu, i), k63 = pick(a.mod.k63, i), ctw = 2ull * comp;
   const uint64_t ct = (uint64_t)blockIdx.x * C, query = ct >> a.log2c;
   const uint32_t k0 = (uint32_t)ct & ((1u << a.log2c) - 1), at = i * n + s;
+  chain_wait();
   if (!FOLD && k0 >= a.olimit) return;
   const uint32_t *in = a.cur + ct * (FOLD ? 2 : 1) * ctw + at;
   const uint64_t in_step = (FOLD ? 2 : 1) * ctw, dh_step = (uint64_t)a.rows * comp;
@@ -248,8 +250,8 @@ cudaError_t digits_launch(const ParamCtx &c, const GadgetConst &g, const uint32_
       if (dev < 64) known.fetch_or(1ull << dev, std::memory_order_acq_rel);
     }
   }
-  kernel<<<(unsigned)polys, kGroups<LOGN, L> * N / 16, smem, s>>>(cur, dig, c.ntt, g, ell, gadget_bits(c.p, ell));
-  return cudaGetLastError();
+  return launch_chained(kernel, (unsigned)polys, kGroups<LOGN, L> * N / 16, smem, s, cur, dig, c.ntt, g, ell,
+                        gadget_bits(c.p, ell));
 }
 
 template <int LOGN, bool FOLD>
@@ -289,10 +291,8 @@ cudaError_t level(const ParamCtx &c, const GadgetConst &g, MacArgs &a, uint64_t 
   // blocks; below, the level is bound by latency and wants the threads
   const dim3 grid((unsigned)cts, L, n / (4 * kMacThreads));
   if (a.log2c >= 1 && cts * L * grid.z >= 152 * 32)
-    k_gadget_mac<FOLD, 2><<<dim3(grid.x / 2, grid.y, grid.z), kMacThreads, 0, s>>>(a);
-  else
-    k_gadget_mac<FOLD, 1><<<grid, kMacThreads, 0, s>>>(a);
-  return cudaGetLastError();
+    return launch_chained(k_gadget_mac<FOLD, 2>, dim3(grid.x / 2, grid.y, grid.z), kMacThreads, 0, s, a);
+  return launch_chained(k_gadget_mac<FOLD, 1>, grid, kMacThreads, 0, s, a);
 }
 
 }  // namespace

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(256) k_slots_to_responses_v(const uint32_t *__
   const uint32_t s0 = blockIdx.y * VT;
   const uint32_t j = s0 >> logn, k0 = s0 & (n - 1);
   const uint32_t t = threadIdx.x, lane16 = t & 15, row = t >> 4;
+  chain_wait();
   for (uint32_t kk = row; kk < VT; kk += 16) {
     const uint64_t f = f0 + 4 * lane16;
     uint4 v = make_uint4(0, 0, 0, 0);
@@ -279,8 +280,7 @@ cudaError_t launch_slots_to_responses(const ParamCtx &c, const uint32_t *out, ui
   const uint64_t F = (uint64_t)2 * B * D2;
   if (F % 4 == 0) {
     dim3 grid((unsigned)((F + VT - 1) / VT), (c.p.L << c.logn) / VT);
-    k_slots_to_responses_v<<<grid, 256, 0, s>>>(out, 2 * B, D2, c.p.L, c.logn, resp);
-    return cudaGetLastError();
+    return launch_chained(k_slots_to_responses_v, grid, 256, 0, s, out, 2 * B, D2, c.p.L, c.logn, resp);
   }
   dim3 grid((unsigned)((F + TF - 1) / TF), (c.p.L << c.logn) / TK);
   k_slots_to_responses<<<grid, 256, 0, s>>>(out, 2 * B, D2, c.p.L, c.logn, resp);

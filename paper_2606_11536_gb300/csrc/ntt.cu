@@ -80,6 +80,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
   constexpr int N = 1 << LOGN;
   extern __shared__ uint32_t sm[];
   const bool wide = wide_ok(dst);
+  chain_wait();
   for (uint32_t row = blockIdx.x; row < rows; row += gridDim.x) {
     const uint32_t p = rm.L.div(row), j = row - p * rm.L.d;
     const uint64_t poly = SRC == SRC_RAW ? rs.poly(p) : 0;
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
   extern __shared__ uint32_t sm[];
   const uint32_t tid = threadIdx.x;
   const bool wide = wide_ok(src);
+  chain_wait();
   for (uint32_t row = blockIdx.x; row < rows; row += gridDim.x) {
     const uint32_t j = rm.L.mod(row);
     const uint32_t q = pick(C.q, j);
@@ -173,6 +175,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN == 13 ? 1 : 12288 >> LOG
   extern __shared__ uint32_t sm[];
   const uint32_t half = threadIdx.x / T, tid = threadIdx.x % T;
   const bool wide = wide_ok(src);
+  chain_wait();
   for (uint32_t r = 0; r < (L + 1) / 2; ++r) {
     const uint32_t j = 2 * r + half;
     const bool act = j < L;  // the barriers below are reached by both halves
@@ -223,6 +226,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8)
   const uint32_t q = pick(C.q, j);
   const uint2 *tw = pick(C.fwd, j);
   const uint32_t *gin = src + (row0 + (uint64_t)i * 2 * L + (uint64_t)half * L + j) * N;
+  chain_wait();
   uint32_t v[16];
   fwd_row<LOGN>(smh, [&](uint32_t i) { return __ldg(gin + i); }, tw, q, tid, v);
   // n = 2^13 reads its neighbours' words in the last pass
@@ -244,10 +248,8 @@ cudaError_t fwd_launch(const ParamCtx &c, const uint32_t *src, const RowMap &rm,
   const size_t smem = ((1u << LOGN) + (1u << LOGN) / 16) * sizeof(uint32_t);
   const unsigned grid = (unsigned)(rows < kMaxGrid ? rows : kMaxGrid);
   if (raw)
-    k_ntt_fwd<LOGN, SRC_RAW><<<grid, T, smem, s>>>(nullptr, rm, rs, dst, c.ntt, (uint32_t)rows);
-  else
-    k_ntt_fwd<LOGN, SRC_U32><<<grid, T, smem, s>>>(src, rm, rs, dst, c.ntt, (uint32_t)rows);
-  return cudaGetLastError();
+    return launch_chained(k_ntt_fwd<LOGN, SRC_RAW>, grid, T, smem, s, nullptr, rm, rs, dst, c.ntt, (uint32_t)rows);
+  return launch_chained(k_ntt_fwd<LOGN, SRC_U32>, grid, T, smem, s, src, rm, rs, dst, c.ntt, (uint32_t)rows);
 }
 
 template <int LOGN>
@@ -256,8 +258,7 @@ cudaError_t inv_launch(const ParamCtx &c, const uint32_t *src, const RowMap &rm,
   const int T = (1 << LOGN) / 16;
   const size_t smem = ((1u << LOGN) + (1u << LOGN) / 16) * sizeof(uint32_t);
   const unsigned grid = (unsigned)(rows < kMaxGrid ? rows : kMaxGrid);
-  k_ntt_inv<LOGN><<<grid, T, smem, s>>>(src, rm, dst, c.ntt, (uint32_t)rows);
-  return cudaGetLastError();
+  return launch_chained(k_ntt_inv<LOGN>, grid, T, smem, s, src, rm, dst, c.ntt, (uint32_t)rows);
 }
 
 cudaError_t fwd_any(const ParamCtx &c, const uint32_t *src, const RowMap &rm, const RawSrc &rs, uint32_t *dst,
@@ -312,8 +313,7 @@ cudaError_t pair_launch(const ParamCtx &c, const uint32_t *src, uint64_t row0, u
   if (smem > 48 * 1024 &&  // above the limit a kernel has without asking
       (e = cudaFuncSetAttribute(k_ntt_fwd_pair_slots<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
     return e;
-  k_ntt_fwd_pair_slots<LOGN><<<kc * c.p.L, T, smem, s>>>(src, row0, c.ntt, c.p.L, stride, col0, slots);
-  return cudaGetLastError();
+  return launch_chained(k_ntt_fwd_pair_slots<LOGN>, kc * c.p.L, T, smem, s, src, row0, c.ntt, c.p.L, stride, col0, slots);
 }
 
 cudaError_t launch_ntt_fwd_pair_slots(const ParamCtx &c, const uint32_t *queries, uint32_t i0, uint32_t kc,
@@ -340,8 +340,9 @@ cudaError_t switch_launch(const ParamCtx &c, const uint32_t *src, uint32_t *dst,
     return e;
   for (uint64_t first = 0; first < count; first += kMaxGrid) {
     const uint64_t nb = count - first < kMaxGrid ? count - first : kMaxGrid;
-    k_ntt_inv_switch<LOGN><<<(unsigned)nb, N / 8, smem, s>>>(src + first * L * N, dst + first * N, c.ntt, c.sw, L);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_chained(k_ntt_inv_switch<LOGN>, (unsigned)nb, N / 8, smem, s, src + first * L * N, dst + first * N,
+                            c.ntt, c.sw, L)) != cudaSuccess)
+      return e;
   }
   return cudaSuccess;
 }

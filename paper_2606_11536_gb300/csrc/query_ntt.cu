@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kCtaThreads, LOGN == 11 ? 2 : 3) k_ntt_query_d
   const auto ciphertext = [&](uint32_t e) {  // of position 8h + e of the 16
     return 16 * u + (IN_ORDER ? 8 * h + e : 4 * h + 2 * (e >> 2) + (e & 1) + 8 * ((e >> 1) & 1));
   };
+  chain_wait();
   const bool any = m < a.M && ciphertext(0) < a.Kc;  // the least of the eight
   const uint32_t slot0 = tid >> 1, dig = 2 * (tid & 1);  // two digits of a slot per thread
   const uint64_t slot_step = (uint64_t)gridDim.y * a.Mp * 64;
@@ -159,8 +160,7 @@ cudaError_t query_launch(const QueryArgs &a, uint32_t Uc, cudaStream_t s) {
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
     if (dev < 64) known.fetch_or(1ull << dev, std::memory_order_acq_rel);
   }
-  kernel<<<dim3((1u << LOGN) / kSlots * 2 * a.Mp, Uc, a.L), kCtaThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(kernel, dim3((1u << LOGN) / kSlots * 2 * a.Mp, Uc, a.L), kCtaThreads, smem, s, a);
 }
 
 template <int LOGN>

@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_scan_direct(ScanArgs a, M
   uint32_t *tile = reinterpret_cast<uint32_t *>(smem);  // [M][cols][kDirectWarps + 1]
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t s0 = blockIdx.x * kDirectWarps, s = s0 + warp;
+  chain_wait();
   const uint32_t c0 = blockIdx.y * kDirectCols, cols = min(kDirectCols, a.D2 - c0), nq = cols >> 2;
   uint32_t QW = 1;
   while (QW < nq) QW <<= 1;
@@ -373,8 +374,7 @@ template <int MB>
 cudaError_t direct_launch(const ParamCtx &c, const ScanArgs &a, cudaStream_t s) {
   const size_t smem = a.out_poly ? (size_t)a.M * kDirectCols * (kDirectWarps + 1) * 4 : 0;  // 36 KiB at most
   const dim3 grid(a.nslots / kDirectWarps, (a.D2 + kDirectCols - 1) / kDirectCols, (a.M + MB - 1) / MB);
-  k_scan_direct<MB><<<grid, kDirectWarps * 32, smem, s>>>(a, c.mod);
-  return cudaGetLastError();
+  return launch_chained(k_scan_direct<MB>, grid, kDirectWarps * 32, smem, s, a, c.mod);
 }
 
 template <int MB, int T>
