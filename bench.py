@@ -360,20 +360,25 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     M = 2 * B
     nslots = L_PRIMES * n
     launch_ms = gemm_ms / launches_per_step
-    streaming = layout == g.PIR_LAYOUT_PLAIN and M <= 8 and (tile in (1, 2, 3, 7) or (tile == 0 and M <= 4 and D2 <= 512))
+    # the digit GEMM: its tile ids, or the default tile (plain: from two queries and 128 rows on)
+    digits = ((layout == g.PIR_LAYOUT_PLAIN and (tile == 9 or (tile == 0 and M >= 3 and D1 >= 128)))
+              or (layout == g.PIR_LAYOUT_LIMB and tile in (0, 4)))
+    streaming = (layout == g.PIR_LAYOUT_PLAIN and not digits and M <= 8
+                 and (tile in (1, 2, 3, 7) or (tile == 0 and M <= 4 and D2 <= 512)))
     if streaming:
         kernel_tag = "scan_tma" if tile in (0, 7) else "gemv_scan"
         alg_bytes = nslots * (D1 * D2 * 4 + D1 * M * 4 + M * D2 * 4)
         per = alg_bytes / launches_per_step
         rl = {"bound": "hbm", "achieved": per / (launch_ms / 1e3) / 1e9, "peak": float(ctx.peaks["hbm_gbs"]),
               "unit": "GB/s", "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % ctx.peak_kind}
-    elif layout == g.PIR_LAYOUT_TENSOR:
-        # bf16 tensor cores: 16 digit products (2 FLOP each) per modular MAC of the
+    elif layout == g.PIR_LAYOUT_TENSOR or digits:
+        # f16 or bf16 tensor cores: 16 digit products (2 FLOP each) per modular MAC of the
         # useful query rows, against the measured sustained dense bf16 peak (the
-        # kernel runs inside a long step); bytes: 8 per DB residue (four bf16 digits)
-        kernel_tag = "gemm_tc"
+        # kernel runs inside a long step); bytes: 8 per DB residue (four bf16 digits) in
+        # the tensor layout, 4 where the digits are made in the kernel
+        kernel_tag = "gemm_digit" if digits else "gemm_tc"
         macs = nslots * D1 * D2 * M / launches_per_step
-        alg_bytes = nslots * (D1 * D2 * 8 + D1 * M * 8 + M * D2 * 4)
+        alg_bytes = nslots * (D1 * D2 * (4 if digits else 8) + D1 * M * 8 + M * D2 * 4)
         per = alg_bytes / launches_per_step
         rl = {"bound": "tensor", "achieved": 32.0 * macs / (launch_ms / 1e3) / 1e12,
               "peak": float(ctx.peaks.get("bf16_tflops_sustained", 1700.0)), "unit": "TFLOP/s",
@@ -409,7 +414,7 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     rl["alg_bytes_per_launch"] = per
     src = os.path.join(ROOT, "paper_2606_11536_gb300", "csrc",
                        {"scan_tma": "scan_tma.cu", "gemv_scan": "gemm_plain.cu", "gemm_plain": "gemm_plain.cu",
-                        "gemm_limb": "gemm_limb.cu", "gemm_tc": "gemm_tc.cu"}[kernel_tag])
+                        "gemm_limb": "gemm_limb.cu", "gemm_tc": "gemm_tc.cu", "gemm_digit": "gemm_digit.cu"}[kernel_tag])
     rl["traffic"] = profile_traffic(kernel_tag, ctx.wl, B, src, launches_per_step)
     return rl
 
@@ -946,7 +951,6 @@ def lwe_bench(args):
           .contiguous() for t in range(nbuf)]
     out = torch.empty(B * D1, dtype=torch.int32, device=dev)
     stream = torch.cuda.current_stream()
-    peak_tops = g.pir_probe_int8_mma(stream)
 
     def step(t):
         g.pir_lwe_answer(db, D1, D0, qs[t % nbuf], B, out, path=path, stream=stream)
@@ -975,11 +979,12 @@ def lwe_bench(args):
     macs = D1 * D0 * B
     peaks, kind = measured_peaks()
     if path == g.PIR_LWE_TENSOR:
-        achieved = 2.0 * 4 * macs / (ms / 1e3) / 1e12  # four byte planes per INT8 x INT32 product
-        roofline = {"bound": "tensor", "achieved": achieved, "peak": peak_tops, "unit": "TOPS (INT8 mma.sync)",
-                    "frac": achieved / peak_tops, "traffic": None, "kernel": "lwe_mma",
-                    "peak_source": "pir_probe_int8_mma on this GPU (MEASURED_PEAKS.json has no INT8 entry)",
-                    "hbm_frac": (raw * -(-B // (16 if B >= 16 else 8)) / (ms / 1e3) / 1e9) / float(peaks["hbm_gbs"])}
+        achieved = 2.0 * 4 * macs / (ms / 1e3) / 1e12  # four f16 digits per INT8 x INT32 product
+        peak = float(peaks.get("bf16_tflops_sustained", 1700.0))
+        roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                    "frac": achieved / peak, "traffic": None, "kernel": "lwe_tc",
+                    "peak_source": "%s bf16_tflops_sustained (MEASURED_PEAKS.json)" % kind,
+                    "hbm_frac": (raw * -(-B // 32) / (ms / 1e3) / 1e9) / float(peaks["hbm_gbs"])}
     else:
         achieved = raw * -(-B // min(B, 4)) / (ms / 1e3) / 1e9  # the DB streams once per group of 4 queries
         roofline = {"bound": "hbm", "achieved": achieved, "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
