@@ -376,7 +376,8 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
         # useful query rows, against the measured sustained dense bf16 peak (the
         # kernel runs inside a long step); bytes: 8 per DB residue (four bf16 digits) in
         # the tensor layout, 4 where the digits are made in the kernel
-        kernel_tag = "gemm_digit" if digits else "gemm_tc"
+        kernel_tag = ("gemm_tc" if not digits else
+                      "gemm_digit" if layout == g.PIR_LAYOUT_PLAIN else "gemm_digit_limb")
         macs = nslots * D1 * D2 * M / launches_per_step
         alg_bytes = nslots * (D1 * D2 * (4 if digits else 8) + D1 * M * 8 + M * D2 * 4)
         per = alg_bytes / launches_per_step
@@ -414,7 +415,8 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     rl["alg_bytes_per_launch"] = per
     src = os.path.join(ROOT, "paper_2606_11536_gb300", "csrc",
                        {"scan_tma": "scan_tma.cu", "gemv_scan": "gemm_plain.cu", "gemm_plain": "gemm_plain.cu",
-                        "gemm_limb": "gemm_limb.cu", "gemm_tc": "gemm_tc.cu", "gemm_digit": "gemm_digit.cu"}[kernel_tag])
+                        "gemm_limb": "gemm_limb.cu", "gemm_tc": "gemm_tc.cu", "gemm_digit": "gemm_digit.cu",
+                        "gemm_digit_limb": "gemm_digit.cu"}[kernel_tag])
     rl["traffic"] = profile_traffic(kernel_tag, ctx.wl, B, src, launches_per_step)
     return rl
 

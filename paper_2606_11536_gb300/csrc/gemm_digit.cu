@@ -45,11 +45,14 @@
 // own row, tcgen05.st.32x32b.)
 //
 // Measured (GB300, 2.07 GHz, against the CUDA-core tiles): 8 GiB DB (n = 4096, 2048 x 512),
-// batch 32: 69.4 -> 12.8 ms, 0.76 of the sustained bf16 rate as 16 digit products; 1 GiB DB
-// (n = 2048, 512 x 512), batch 8: 2.3 -> 0.83 ms, 5.2 TB/s of DB words; 1 GiB DB (n = 4096),
+// batch 32: 69.4 -> 12.2 ms, 0.85 of the sustained bf16 rate as 16 digit products; 1 GiB DB
+// (n = 2048, 512 x 512), batch 8: 2.3 -> 0.81 ms, 5.3 TB/s of DB words; 1 GiB DB (n = 4096),
 // batch 4: 1.38 -> 0.73 ms; limb layout (n = 2048, 512 x 256), batch 32: 7.8 (INT8 mma.sync) ->
-// 1.4 ms.  With few query rows it is bound by HBM, from 2B = 32 by the
-// MMAs (and, where D1 is short, by the epilogue's serial parts).
+// 0.89 ms.  With few query rows it is bound by HBM, from 2B = 32 by the
+// MMAs (and, where D1 is short, by the epilogue's serial parts).  Handing the accumulators back
+// before the arithmetic on their copies took the limb case from 1.00 ms there, the 8 GiB one
+// from 12.8.  The second half's MMAs one stage behind the first's, so that the next unit's first
+// half would not wait at all, were slower (16.3 ms): the A ring loses the slot its converters need.
 //
 // Every barrier wait is bounded; one that runs out sets the device error word.
 #include "async.cuh"
@@ -483,15 +486,30 @@ __global__ void __launch_bounds__(kThreads, 1)
             fence_after();
           }
           const uint32_t item = set + kSets * (it % kPer);
+          uint32_t f[4][8];
           if (item < items) {  // two groups in flight; a missing second one is the first again
             const uint32_t src = tmem + rt.slot * a.W + ((32 * quarter) << 16) + 16 * item;
             const uint32_t src2 = item + kSets < items ? src + 16 * kSets : src;
-            uint32_t f[4][8];
             tmem_ld_16x256b_x2(src, f[0]);
             tmem_ld_16x256b_x2(src + (16 << 16), f[1]);
             tmem_ld_16x256b_x2(src2, f[2]);
             tmem_ld_16x256b_x2(src2 + (16 << 16), f[3]);
             tmem_ld_wait(f[0], f[1], f[2], f[3]);
+          }
+          // the accumulators are handed back before the arithmetic on their copies: the next
+          // unit's MMAs wait for them
+          if (it % kPer == kPer - 2) {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if (CG == 2)
+                mbar_arrive_at(tempty_lead + 8 * rt.slot);
+              else
+                mbar_arrive(tempty + 8 * rt.slot);
+            }
+            rt.next(a.R);
+          }
+          if (item < items) {
 #pragma unroll
             for (int g2 = 0; g2 < 2; ++g2) {
               int64_t sum[2];
@@ -509,17 +527,6 @@ __global__ void __launch_bounds__(kThreads, 1)
               // 16 products of 2^24 * 2^30 a chunk: below 2^62 after 16 chunks
               tot[it + g2] += (p ? sum[1] : sum[0]) + __shfl_xor_sync(0xffffffffu, p ? sum[0] : sum[1], 1);
             }
-          }
-          if (it % kPer == kPer - 2) {
-            fence_before();
-            __syncwarp();
-            if (lane == 0) {
-              if (CG == 2)
-                mbar_arrive_at(tempty_lead + 8 * rt.slot);
-              else
-                mbar_arrive(tempty + 8 * rt.slot);
-            }
-            rt.next(a.R);
           }
         }
       }
