@@ -383,8 +383,9 @@ pir_status_t pir_answer_folded(pir_db_t db, const uint32_t *queries, uint32_t B,
  * (tcgen05 f16, signed digits, exact 1024-byte f32 sums; the query digits take scratch
  * from the stream-ordered allocator, 8 bytes per query word, without which the
  * CUDA-core path answers), PIR_LWE_SIMT (CUDA-core dp4a on byte planes), or
- * PIR_LWE_AUTO (the faster of the two for these sizes).  D0 must be a multiple of 16
- * and at most 2^24; buffers 16-byte aligned.  Asynchronous on stream; the caller owns
+ * PIR_LWE_AUTO (the faster of the two for these sizes).  The CUDA-core path answers
+ * databases of more than 2^31 rows, which tensor maps do not reach.  D0 must be a multiple
+ * of 16 and at most 2^24; buffers 16-byte aligned.  Asynchronous on stream; the caller owns
  * every buffer.
  * Errors: PIR_ERR_ARG (NULL or misaligned buffers, zero or unsupported sizes, unknown
  * path), PIR_ERR_CUDA. */
@@ -393,6 +394,10 @@ pir_status_t pir_answer_folded(pir_db_t db, const uint32_t *queries, uint32_t B,
 #define PIR_LWE_SIMT 2u
 pir_status_t pir_lwe_answer(const int8_t *db, uint32_t D1, uint32_t D0, const uint32_t *queries, uint32_t B,
                             uint32_t *out, uint32_t path, void *stream);
+/* The path (PIR_LWE_TENSOR or PIR_LWE_SIMT) that pir_lwe_answer takes for `path` at these
+ * sizes, where memory for its scratch can be had.  Host arithmetic only.
+ * Errors: PIR_ERR_ARG (NULL, zero sizes, unknown path). */
+pir_status_t pir_lwe_path(uint32_t D1, uint32_t D0, uint32_t B, uint32_t path, uint32_t *taken);
 
 /* Measured peak of the INT8 warp-level tensor instruction (mma.sync m16n8k32 s8 x u8
  * -> s32) on the current device, in tera-operations per second (2 per multiply-add):

@@ -97,6 +97,7 @@ def lib():
             "pir_autotune": (i32, [vp, u32, vp, u32, C.POINTER(pir_answer_opts_t)]),
             "pir_answer_noalloc": (i32, [vp, vp, u32, vp, vp]),
             "pir_lwe_answer": (i32, [vp, u32, u32, vp, u32, vp, u32, vp]),
+            "pir_lwe_path": (i32, [u32, u32, u32, u32, C.POINTER(u32)]),
             "pir_fold": (i32, [P, vp, u32, u32, u32, vp, vp, vp]),
             "pir_answer_folded": (i32, [vp, vp, u32, u32, vp, vp, i32, vp, C.POINTER(pir_answer_opts_t)]),
             "pir_probe_int8_mma": (i32, [vp, C.POINTER(C.c_double)]),
@@ -317,6 +318,13 @@ def pir_lwe_answer(db, D1: int, D0: int, queries, B: int, out, path: int = PIR_L
         raise ValueError("pir_lwe_answer works on device buffers")
     _check(lib().pir_lwe_answer(dp, D1, D0, qp, B, op, path, _stream_ptr(stream)), "pir_lwe_answer")
     return out
+
+
+def pir_lwe_path(D1: int, D0: int, B: int, path: int = PIR_LWE_AUTO) -> int:
+    """The path that pir_lwe_answer takes for `path` at these sizes (host arithmetic only)."""
+    v = C.c_uint32()
+    _check(lib().pir_lwe_path(D1, D0, B, path, C.byref(v)), "pir_lwe_path")
+    return int(v.value)
 
 
 def pir_probe_int8_mma(stream=None) -> float:

@@ -174,6 +174,7 @@ cudaError_t launch_gemm_plain(const ParamCtx &c, const uint32_t *db, uint32_t D1
 uint32_t gemm_plain_tiles();
 
 // lwe_tc.cu: the scalar-HE product on the tensor cores; qt is scratch for the query digits.
+bool lwe_tc_addresses(uint32_t D1);  // whether its tensor maps reach all rows of the DB
 size_t lwe_tc_scratch_bytes(uint32_t D0, uint32_t B);
 cudaError_t launch_lwe_tc(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
                           uint16_t *qt, cudaStream_t s);

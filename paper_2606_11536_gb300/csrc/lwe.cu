@@ -135,7 +135,7 @@ cudaError_t dp4a_launch(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_
   constexpr int smem = 2 * (256 * KS + QB * KS * 4) + QB * KS * 4;
   cudaError_t e = cudaFuncSetAttribute(k_lwe_dp4a<QB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const uint64_t gx = (D1 + 255) / 256, gy = (B + QB - 1) / QB;
+  const uint64_t gx = (D1 + 255ull) / 256, gy = (B + QB - 1) / QB;
   if (gx > 0x7FFFFFFFull || gy > 65535) return cudaErrorInvalidConfiguration;
   // split K until the grid fills about four waves of resident CTAs
   int dev = 0, sms = 0, per_sm = 0;
@@ -173,12 +173,18 @@ bool tensor_path_wins(uint32_t D1, uint32_t D0, uint32_t B) {
   return gain_us >= 7 || (D0 >= 1024 && (B >= 4 || (B == 3 && gain_us >= 3)));
 }
 
+// The path that `path` stands for at these sizes: the tensor cores only where their tensor maps
+// reach every row.
+uint32_t lwe_path(uint32_t D1, uint32_t D0, uint32_t B, uint32_t path) {
+  if (path == PIR_LWE_AUTO) path = tensor_path_wins(D1, D0, B) ? PIR_LWE_TENSOR : PIR_LWE_SIMT;
+  return path == PIR_LWE_TENSOR && !lwe_tc_addresses(D1) ? PIR_LWE_SIMT : path;
+}
+
 // The tensor path takes scratch for the query digits; where there is none left, or the
 // runtime offers no tensor maps, the CUDA cores answer.
 cudaError_t launch_lwe_gemm(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
                             uint32_t path, cudaStream_t s, uint32_t *launches) {
-  if (path == PIR_LWE_AUTO) path = tensor_path_wins(D1, D0, B) ? PIR_LWE_TENSOR : PIR_LWE_SIMT;
-  if (path == PIR_LWE_TENSOR && tensor_maps_available()) {
+  if (lwe_path(D1, D0, B, path) == PIR_LWE_TENSOR && tensor_maps_available()) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -212,5 +218,11 @@ extern "C" pir_status_t pir_lwe_answer(const int8_t *db, uint32_t D1, uint32_t D
   cudaError_t e = launch_lwe_gemm(db, D1, D0, queries, B, out, path, static_cast<cudaStream_t>(stream), &launches);
   if (e != cudaSuccess) return cuda_status(e);
   count_launches(launches);
+  return PIR_OK;
+}
+
+extern "C" pir_status_t pir_lwe_path(uint32_t D1, uint32_t D0, uint32_t B, uint32_t path, uint32_t *taken) {
+  if (!taken || D1 == 0 || D0 == 0 || B == 0 || path > PIR_LWE_SIMT) return PIR_ERR_ARG;
+  *taken = gbpir::lwe_path(D1, D0, B, path);
   return PIR_OK;
 }

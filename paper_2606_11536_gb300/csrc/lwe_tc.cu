@@ -372,10 +372,15 @@ uint32_t padded_words(uint32_t D0) { return (D0 + kK - 1) / kK * kK; }
 
 }  // namespace
 
+// Tensor-map coordinates are signed 32-bit: the last row of the last tile has to lie below
+// 2^31 (tiles of 256 rows where CTAs work in pairs).  Past it a box reads as zeros.
+bool lwe_tc_addresses(uint32_t D1) { return (D1 + 255ull) / 256 * 256 <= 1ull << 31; }
+
 size_t lwe_tc_scratch_bytes(uint32_t D0, uint32_t B) { return (size_t)padded_words(D0) * padded_queries(B) * 8; }
 
 cudaError_t launch_lwe_tc(const int8_t *A, uint32_t D1, uint32_t D0, const uint32_t *Q, uint32_t B, uint32_t *out,
                           uint16_t *qt, cudaStream_t s) {
+  if (!lwe_tc_addresses(D1)) return cudaErrorInvalidValue;
   LweArgs a = {};
   cudaError_t e = device_error_word(&a.err);
   if (e != cudaSuccess) return e;
