@@ -140,8 +140,7 @@ typedef struct {
                         rows padded to 16 to be multiples of 32 and 64 (limb 4, the
                         f16 tensor-core GEMM, is the built-in choice); tensor 1 is
                         the 1-SM GEMM, 2 the CTA-pair (2-SM) GEMM, which needs
-                        D2 % 64 == 0, 3 and 4 the 1-SM GEMM in clusters of 2 and 4
-                        CTAs that multicast the query digits, which need D2 % 64
+                        D2 % 64 == 0, 3 and 4 stand for tensor 1 and need D2 % 64
                         and D2 % 128 == 0, 5 the CTA-pair GEMM loading by tensor
                         maps, which needs D2 % 64 == 0 and the query rows padded to
                         8 (Mp) with 4 Mp <= 256 or a multiple of 256; otherwise

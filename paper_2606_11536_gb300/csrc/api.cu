@@ -1463,8 +1463,7 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
   const bool limb = db->layout == PIR_LAYOUT_LIMB;
   std::vector<uint32_t> tiles;
   if (db->layout == PIR_LAYOUT_TENSOR) {
-    tiles.push_back(1);
-    for (uint32_t t = 2; t <= gemm_tc_tiles(); ++t)
+    for (uint32_t t : {1u, 2u, 5u})  // (3 and 4 are form 1)
       if (gemm_tc_tile_ok(t, layout_rows(db->layout, M), p.D2)) tiles.push_back(t);
   } else if (!limb) {
     if (M <= 2) tiles.push_back(1);
