@@ -277,6 +277,13 @@ struct FastDiv {
 // (whose blocks fill the SMs only once all of this kernel's have begun).  The gap it closes is 1 to
 // 2 us a launch: smallest answer (three launches) 18.8 -> 15.5 us, 26 folding launches 432 -> 380,
 // expansion of one query by 16 108 -> 73 us, 1001 inverse rows x 3 of n = 2^13 67.6 -> 64.8.
+//
+// Such a kernel is resident while its input is still being written.  So it reads what another
+// kernel of the stream may have written by plain loads through pointers without __restrict__:
+// __ldg (ld.global.nc) is defined for memory that nobody writes while the kernel lives, and the
+// compiler may move it, or any access through a __restrict__ pointer, above the wait.  __ldg
+// stays for tables, keys and the resident DB: two launches back or more, they are complete
+// before this kernel can start.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");

@@ -37,7 +37,7 @@ struct ScaleConst {
 };
 
 // x * 2^-levels for every residue of rows [rows][n]: block = one row, row r under prime r % L.
-__global__ void k_expand_scale(uint32_t *__restrict__ x, uint32_t n, uint32_t L, ScaleConst E) {
+__global__ void k_expand_scale(uint32_t *x, uint32_t n, uint32_t L, ScaleConst E) {
   const uint32_t i = blockIdx.x % L;
   uint32_t q = E.q[0], w = E.inv2l[0], wsh = E.inv2l_sh[0];
 #pragma unroll

@@ -26,8 +26,13 @@
 namespace gbpir {
 namespace {
 
+// ldg4: of tables and keys only (chain_wait)
 __device__ __forceinline__ void ldg4(uint32_t (&v)[4], const uint32_t *p) {
   const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p));
+  v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+}
+__device__ __forceinline__ void ld4(uint32_t (&v)[4], const uint32_t *p) {
+  const uint4 x = *reinterpret_cast<const uint4 *>(p);
   v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
 }
 __device__ __forceinline__ void st4(uint32_t *p, const uint32_t (&v)[4]) {
@@ -67,8 +72,7 @@ constexpr uint32_t kGroups = L < (16384u >> LOGN) ? L : (16384u >> LOGN);
 template <int LOGN, uint32_t L, bool FOLD>
 __global__ void __launch_bounds__(kGroups<LOGN, L> << (LOGN - 4),
                                   (kGroups<LOGN, L> << (LOGN - 4)) > 768 ? 1 : 1536 / (kGroups<LOGN, L> << (LOGN - 4)))
-    k_gadget_digits(const uint32_t *__restrict__ cur, uint32_t *__restrict__ dig, NttConst C, GadgetConst g,
-                    uint32_t ell, uint32_t w) {
+    k_gadget_digits(const uint32_t *cur, uint32_t *dig, NttConst C, GadgetConst g, uint32_t ell, uint32_t w) {
   constexpr uint32_t N = 1u << LOGN, PADN = N + N / 16, T = N / 16, G = kGroups<LOGN, L>;
   extern __shared__ uint32_t sm[];
   const uint32_t grp = threadIdx.x / T, tid = threadIdx.x % T;
@@ -154,8 +158,8 @@ __global__ void __launch_bounds__(kMacThreads) k_gadget_mac(const MacArgs a) {
   uint32_t va[C][4], vb[C][4], p[4];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    ldg4(va[c], in + c * in_step);
-    ldg4(vb[c], in + c * in_step + comp);
+    ld4(va[c], in + c * in_step);
+    ld4(vb[c], in + c * in_step + comp);
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc_a[c][e] = FOLD ? va[c][e] : 0, acc_b[c][e] = FOLD ? vb[c][e] : 0;
   }
@@ -171,10 +175,10 @@ __global__ void __launch_bounds__(kMacThreads) k_gadget_mac(const MacArgs a) {
     for (int c = 0; c < C; ++c) {
       uint32_t d[4];
       if (FOLD) {
-        ldg4(d, dh + c * dh_step);
+        ld4(d, dh + c * dh_step);
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) d[e] = __ldg(dh + c * dh_step + p[e]);
+        for (int e = 0; e < 4; ++e) d[e] = dh[c * dh_step + p[e]];
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -191,10 +195,14 @@ __global__ void __launch_bounds__(kMacThreads) k_gadget_mac(const MacArgs a) {
         for (int e = 0; e < 4; ++e) acc_a[c][e] = fold63(acc_a[c][e], k63), acc_b[c][e] = fold63(acc_b[c][e], k63);
     }
   }
-  uint32_t m[4], msh[4];
+  uint32_t m[4], msh[4], bp[C][4];  // bp: b[p] of all C, read before the first output is written
   if (!FOLD) {
     ldg4(m, a.mon + at);
     ldg4(msh, a.mon_sh + at);
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) bp[c][e] = a.cur[(ct + c) * ctw + comp + i * n + p[e]];
   }
 #pragma unroll
   for (int c = 0; c < C; ++c) {
@@ -208,11 +216,10 @@ __global__ void __launch_bounds__(kMacThreads) k_gadget_mac(const MacArgs a) {
     } else {
       if (k0 + c >= a.olimit) return;
       uint32_t *o = a.out + (query * a.ostride + k0 + c) * ctw + at;
-      const uint32_t *bp = a.cur + (ct + c) * ctw + comp + i * n;
       uint32_t o0[4], o1[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        sb[e] = csub(__ldg(bp + p[e]) + sb[e], q);  // b[p] + S_b
+        sb[e] = csub(bp[c][e] + sb[e], q);  // b[p] + S_b
         o0[e] = csub(va[c][e] + sa[e], q);
         o1[e] = csub(vb[c][e] + sb[e], q);
       }

@@ -153,9 +153,8 @@ __global__ void __launch_bounds__(256) k_query_to_slots_v(const uint32_t *__rest
 }
 
 // out[s][f], f = m*D2 + c -> resp[b][c][comp][j][k]; needs M*D2 % 4 == 0.
-__global__ void __launch_bounds__(256) k_slots_to_responses_v(const uint32_t *__restrict__ out, uint32_t M,
-                                                              uint32_t D2, uint32_t L, uint32_t logn,
-                                                              uint32_t *__restrict__ resp) {
+__global__ void __launch_bounds__(256) k_slots_to_responses_v(const uint32_t *out, uint32_t M, uint32_t D2,
+                                                              uint32_t L, uint32_t logn, uint32_t *resp) {
   __shared__ uint32_t tile[VT][VT + 1];  // [k][f]
   const uint32_t n = 1u << logn;
   const uint64_t F = (uint64_t)M * D2;

@@ -64,7 +64,7 @@ __device__ __forceinline__ uint32_t raw_coeff(const RawSrc &rs, uint64_t poly, u
   const uint64_t byte0 = bit0 >> 3;
   const uint32_t nbytes = (uint32_t)(((bit0 & 7) + rs.log2p + 7) >> 3);
   uint64_t w = 0;
-  for (uint32_t b = 0; b < nbytes; ++b) w |= (uint64_t)__ldg(rs.raw + byte0 + b) << (8 * b);
+  for (uint32_t b = 0; b < nbytes; ++b) w |= (uint64_t)rs.raw[byte0 + b] << (8 * b);
   return (uint32_t)((w >> (bit0 & 7)) & ((1ull << rs.log2p) - 1));
 }
 
@@ -75,8 +75,7 @@ constexpr int kNttCtas = LOGN == 13 ? 3 : 20480 >> LOGN;
 
 template <int LOGN, int SRC>
 __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
-    k_ntt_fwd(const uint32_t *__restrict__ src, RowMap rm, RawSrc rs, uint32_t *__restrict__ dst, NttConst C,
-              uint32_t rows) {
+    k_ntt_fwd(const uint32_t *src, RowMap rm, RawSrc rs, uint32_t *dst, NttConst C, uint32_t rows) {
   constexpr int N = 1 << LOGN;
   extern __shared__ uint32_t sm[];
   const bool wide = wide_ok(dst);
@@ -86,7 +85,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
     const uint64_t poly = SRC == SRC_RAW ? rs.poly(p) : 0;
     uint32_t v[16];
     const uint32_t *gin = SRC == SRC_U32 ? src + rm(row) * N : nullptr;
-    const auto load = [&](uint32_t i) { return SRC == SRC_U32 ? __ldg(gin + i) : raw_coeff(rs, poly, i, LOGN); };
+    const auto load = [&](uint32_t i) { return SRC == SRC_U32 ? gin[i] : raw_coeff(rs, poly, i, LOGN); };
     fwd_row<LOGN>(sm, load, pick(C.fwd, j), pick(C.q, j), threadIdx.x, v);
     store16(dst + (uint64_t)row * N + 16 * threadIdx.x, v, wide);
     if (row + gridDim.x < rows) __syncthreads();  // the next row reuses shared memory
@@ -95,7 +94,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
 
 template <int LOGN>
 __global__ void __launch_bounds__((1 << LOGN) / 16, kNttCtas<LOGN>)
-    k_ntt_inv(const uint32_t *__restrict__ src, RowMap rm, uint32_t *__restrict__ dst, NttConst C, uint32_t rows) {
+    k_ntt_inv(const uint32_t *src, RowMap rm, uint32_t *dst, NttConst C, uint32_t rows) {
   constexpr int N = 1 << LOGN;
   extern __shared__ uint32_t sm[];
   const uint32_t tid = threadIdx.x;
@@ -169,8 +168,7 @@ __device__ __forceinline__ uint32_t switch_coeff(const uint32_t *sm, uint32_t pa
 // all threads switch the coefficients, four per 16-byte store.
 template <int LOGN>
 __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN == 13 ? 1 : 12288 >> LOGN)  // 1024 or 1536 threads per SM
-    k_ntt_inv_switch(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst, NttConst C, SwitchConst W,
-                     uint32_t L) {
+    k_ntt_inv_switch(const uint32_t *src, uint32_t *dst, NttConst C, SwitchConst W, uint32_t L) {
   constexpr int N = 1 << LOGN, PADN = N + N / 16, T = N / 16;
   extern __shared__ uint32_t sm[];
   const uint32_t half = threadIdx.x / T, tid = threadIdx.x % T;
@@ -216,8 +214,8 @@ __global__ void __launch_bounds__((1 << LOGN) / 8, LOGN == 13 ? 1 : 12288 >> LOG
 // transforms one row in its own shared buffer, then all threads write the pairs.
 template <int LOGN>
 __global__ void __launch_bounds__((1 << LOGN) / 8)
-    k_ntt_fwd_pair_slots(const uint32_t *__restrict__ src, uint64_t row0, NttConst C, uint32_t L, uint32_t stride,
-                         uint32_t col0, uint32_t *__restrict__ slots) {
+    k_ntt_fwd_pair_slots(const uint32_t *src, uint64_t row0, NttConst C, uint32_t L, uint32_t stride, uint32_t col0,
+                         uint32_t *slots) {
   constexpr int N = 1 << LOGN, PADN = N + N / 16, T = N / 16;
   extern __shared__ uint32_t sm[];
   const uint32_t i = blockIdx.x / L, j = blockIdx.x % L;
@@ -228,7 +226,7 @@ __global__ void __launch_bounds__((1 << LOGN) / 8)
   const uint32_t *gin = src + (row0 + (uint64_t)i * 2 * L + (uint64_t)half * L + j) * N;
   chain_wait();
   uint32_t v[16];
-  fwd_row<LOGN>(smh, [&](uint32_t i) { return __ldg(gin + i); }, tw, q, tid, v);
+  fwd_row<LOGN>(smh, [&](uint32_t i) { return gin[i]; }, tw, q, tid, v);
   // n = 2^13 reads its neighbours' words in the last pass
   __syncwarp();
 #pragma unroll

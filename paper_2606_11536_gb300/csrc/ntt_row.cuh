@@ -42,9 +42,10 @@ __device__ __forceinline__ T pick(const T (&a)[PIR_MAX_L], uint32_t j) {
 
 // 32 bytes at once (a whole sector per thread; the address 32-byte aligned)
 __device__ __forceinline__ void ld_global32(const uint32_t *p, uint32_t *v) {
-  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "l"(p));
+               : "l"(p)
+               : "memory");
 }
 __device__ __forceinline__ void st_global32(uint32_t *p, const uint32_t *v) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
@@ -52,19 +53,19 @@ __device__ __forceinline__ void st_global32(uint32_t *p, const uint32_t *v) {
                : "memory");
 }
 // 16 consecutive words of a row: rows start on 16-byte boundaries only
-__device__ __forceinline__ void load16(const uint32_t *__restrict__ p, uint32_t (&v)[16], bool wide) {
+__device__ __forceinline__ void load16(const uint32_t *p, uint32_t (&v)[16], bool wide) {
   if (wide) {
     ld_global32(p, v);
     ld_global32(p + 8, v + 8);
   } else {
 #pragma unroll
     for (int e = 0; e < 16; e += 4) {
-      const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p + e));
+      const uint4 x = *reinterpret_cast<const uint4 *>(p + e);
       v[e] = x.x, v[e + 1] = x.y, v[e + 2] = x.z, v[e + 3] = x.w;
     }
   }
 }
-__device__ __forceinline__ void store16(uint32_t *__restrict__ p, const uint32_t (&v)[16], bool wide) {
+__device__ __forceinline__ void store16(uint32_t *p, const uint32_t (&v)[16], bool wide) {
   if (wide) {
     st_global32(p, v);
     st_global32(p + 8, v + 8);

@@ -42,12 +42,12 @@ __device__ __forceinline__ uint32_t bfly_half(uint32_t x, uint32_t y, uint2 p, b
 
 // Bits LOGN - 1 .. LOGN - 4 of unit lo, the 16 >> (LOGN - 11) outputs among slots 2048 part ...
 template <int LOGN>
-__device__ __forceinline__ void first_pass(uint32_t *row, const uint32_t *__restrict__ src, bool valid, uint32_t part,
+__device__ __forceinline__ void first_pass(uint32_t *row, const uint32_t *src, bool valid, uint32_t part,
                                            uint32_t lo, const uint2 *__restrict__ tw, uint32_t q) {
   constexpr int BLO = LOGN - 4, TOP = LOGN - 11, OUT = 16 >> TOP;
   uint32_t v[16];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) v[e] = valid ? __ldg(src + lo + ((uint32_t)e << BLO)) : 0u;
+  for (int e = 0; e < 16; ++e) v[e] = valid ? src[lo + ((uint32_t)e << BLO)] : 0u;
 #pragma unroll
   for (int t = 0; t < TOP; ++t) {
     const uint2 p = __ldg(tw + (1u << t) + (part >> (TOP - t)));

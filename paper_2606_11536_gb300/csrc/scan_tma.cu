@@ -303,12 +303,12 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_scan_direct(ScanArgs a, M
       const uint32_t r = r0 + u * PH, rc = r < a.Kc ? r : a.Kc - 1;
       d[u] = __ldg(reinterpret_cast<const uint4 *>(db + (uint64_t)rc * a.D2));
       if constexpr (MB == 2) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(qs + rc * a.Mp));
+        const uint2 v = *reinterpret_cast<const uint2 *>(qs + rc * a.Mp);
         qrow[u][0] = v.x, qrow[u][1] = v.y;
       } else {
 #pragma unroll
         for (int m = 0; m < MB; m += 4) {
-          const uint4 v = m < (int)M ? __ldg(reinterpret_cast<const uint4 *>(qs + rc * a.Mp + m)) : make_uint4(0, 0, 0, 0);
+          const uint4 v = m < (int)M ? *reinterpret_cast<const uint4 *>(qs + rc * a.Mp + m) : make_uint4(0, 0, 0, 0);
           qrow[u][m] = v.x, qrow[u][m + 1] = v.y, qrow[u][m + 2] = v.z, qrow[u][m + 3] = v.w;
         }
       }
