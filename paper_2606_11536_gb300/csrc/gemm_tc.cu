@@ -260,10 +260,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(TcArgs a, ModConst mc) 
           }
         }
       }
-      // drain: never leave with copies in flight
+      // drain: never leave with copies in flight, nor with a commit on its way to this CTA
       const uint32_t first = it > a.S ? it - a.S : 0;
-      for (uint32_t k = first; k < it; ++k)
+      for (uint32_t k = first; k < it; ++k) {
         if (!wait_bounded(full0 + 8 * (k % a.S), (k / a.S) & 1)) atomicExch(a.err, 1u);
+        if (!wait_bounded(empty0 + 8 * (k % a.S), (k / a.S) & 1)) atomicExch(a.err, 1u);
+      }
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
@@ -556,11 +558,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       // drain: never leave with copies in flight (in the TMA form the even CTA's
       // barriers count both CTAs' bytes; the odd CTA's copies are complete once the
-      // even CTA has drained, before the closing cluster barrier)
+      // even CTA has drained, before the closing cluster barrier), nor with one of the
+      // pair's commits on its way to this CTA's barriers: it would arrive in the shared
+      // memory of whichever CTA runs here next
       const uint32_t first = it > a.S ? it - a.S : 0;
-      if (!TMA || rank == 0)
-        for (uint32_t k = first; k < it; ++k)
-          if (!wait_bounded(full0 + 8 * (k % a.S), (k / a.S) & 1)) atomicExch(a.err, 1u);
+      for (uint32_t k = first; k < it; ++k) {
+        if ((!TMA || rank == 0) && !wait_bounded(full0 + 8 * (k % a.S), (k / a.S) & 1)) atomicExch(a.err, 1u);
+        if (!wait_bounded(empty0 + 8 * (k % a.S), (k / a.S) & 1)) atomicExch(a.err, 1u);
+      }
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {

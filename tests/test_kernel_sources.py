@@ -68,3 +68,22 @@ def test_kernels_launched_early_read_their_input_by_plain_loads():
     assert set(non_coherent(first)) <= {"tw"} and "const uint32_t *__restrict__" not in first
     raw = text(os.path.join(CSRC, "ntt.cu"))
     assert "__ldg" not in body(raw, raw.index("raw_coeff("))
+
+
+def test_stage_releases_are_waited_for_before_a_cta_leaves():
+    """An MMA commit arrives on its barrier some time after it was issued, with a pair in both CTAs.
+    Every barrier that releases a stage is waited for after the last stage (the completed phase,
+    where a refill waits for the one before: parity ^ 1), in both CTAs, before the kernel ends."""
+    kernels = 0
+    for path in SOURCES:
+        s = text(path)
+        for m in re.finditer(r"__global__", s):
+            kernel = body(s, m.start())
+            released = set(re.findall(r"commit(?:_pair)?(?:<CG>)?\((empty\w*) \+", kernel))
+            kernels += bool(released)
+            for bar in released:
+                waits = [w.split(";")[0].split("{")[0] for w in re.findall(r"if \(([^\n]*)", kernel) + re.findall(
+                    r"(\w+ = __all_sync[^\n]*)", kernel) if "wait_bounded(" + bar in w or "wait_bounded(empty " in w]
+                drained = [w for w in waits if "^ 1" not in w]
+                assert any("rank == 0" not in w for w in drained), (re.search(r"k_\w+", kernel).group(0), bar, waits)
+    assert kernels == 4
