@@ -31,8 +31,8 @@ def _sources():
 
 
 def _deps():
-    return (_sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(INCLUDE, "gbpir.h"),
-            os.path.join(CSRC, "exports.map"), os.path.abspath(__file__)])
+    return (_sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
+            + [os.path.join(INCLUDE, "gbpir.h"), os.path.join(CSRC, "exports.map"), os.path.abspath(__file__)])
 
 
 def _compile(src: str, extra: list) -> str:

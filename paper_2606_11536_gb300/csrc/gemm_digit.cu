@@ -57,6 +57,7 @@
 // Every barrier wait is bounded; one that runs out sets the device error word.
 #include "async.cuh"
 #include "common.cuh"
+#include "stage_drain.h"
 #include "tcgen.cuh"
 
 #include <type_traits>
@@ -282,12 +283,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive(fullA + 8 * ra.slot);
       }
     }
-    // the MMAs have read the ring's last stages: no commit is still on its way here
-    if (ok && stages > group) {
-      const uint64_t g = stages - 1 - (stages - 1 - group) % groups;  // this group's last
-      if (g + a.SA >= stages)
-        ok = __all_sync(0xffffffffu, wait_bounded(emptyA + 8 * (uint32_t)(g % a.SA), (uint32_t)(g / a.SA) & 1));
-    }
+    // the MMAs have read the ring's last stages: no commit is still on its way here (with fewer
+    // groups than slots, a group has several of those)
+    for (uint64_t g = first_undrained(stages, group, groups, a.SA); ok && g < stages; g += groups)
+      ok = __all_sync(0xffffffffu, wait_bounded(emptyA + 8 * (uint32_t)(g % a.SA), (uint32_t)(g / a.SA) & 1));
     if (!ok && lane == 0) atomicExch(a.err, 1u);
   } else if (warp == kDbWarp) {
     // ---------------- DB words ----------------

@@ -31,6 +31,7 @@
 // Every barrier wait is bounded; one that runs out sets the device error word.
 #include "async.cuh"
 #include "common.cuh"
+#include "stage_drain.h"
 #include "tcgen.cuh"
 
 #include <cuda_fp16.h>
@@ -173,11 +174,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive(fullA + 8 * ra.slot);
       }
     }
-    // the MMAs have read this group's last stage: no commit is still on its way here
-    if (ok && stages > group) {
-      const uint64_t g = stages - 1 - (stages - 1 - group) % kGroups;
+    // the MMAs have read the ring's last stages: no commit is still on its way here
+    for (uint64_t g = first_undrained(stages, group, kGroups, kSA); ok && g < stages; g += kGroups)
       ok = __all_sync(0xffffffffu, wait_bounded(emptyA + 8 * (uint32_t)(g % kSA), (uint32_t)(g / kSA) & 1));
-    }
     if (!ok && lane == 0) atomicExch(a.err, 1u);
   } else if (warp == kDbWarp || warp == kQueryWarp) {
     // ---------------- DB bytes, query digits ----------------
