@@ -183,6 +183,17 @@ cudaError_t malloc_async_retry(void **ptr, size_t bytes, cudaStream_t s) {
   return e;
 }
 
+// `bytes`, or where the device has no room for them the fewer `tight` (whether it was those:
+// *took_tight).
+cudaError_t malloc_async_either(void **ptr, size_t bytes, size_t tight, cudaStream_t s, bool *took_tight) {
+  *took_tight = false;
+  const cudaError_t e = malloc_async_retry(ptr, bytes, s);
+  if (e != cudaErrorMemoryAllocation || tight >= bytes) return e;
+  cudaGetLastError();
+  *took_tight = true;
+  return malloc_async_retry(ptr, tight, s);
+}
+
 // Device scratch drawn from the stream-ordered allocator; freed (stream-ordered)
 // when the guard goes out of scope.
 struct Scratch {
@@ -190,6 +201,9 @@ struct Scratch {
   cudaStream_t s;
   explicit Scratch(cudaStream_t st) : s(st) {}
   cudaError_t alloc(size_t bytes) { return malloc_async_retry(&ptr, bytes, s); }
+  cudaError_t alloc_either(size_t bytes, size_t tight, bool *took_tight) {
+    return malloc_async_either(&ptr, bytes, tight, s, took_tight);
+  }
   ~Scratch() {
     if (ptr) cudaFreeAsync(ptr, s);
   }
@@ -242,6 +256,28 @@ QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, ui
   const uint32_t rows = gemm_digit_rows(nslots, Kc, round4(M), tight);
   const size_t d = gemm_digit_query_bytes(nslots, rows, round4(M));
   return {d > b ? d : b, rows};
+}
+// Whether the forward NTT of a chunk of kc ciphertexts writes the GEMM's digits itself
+// (digit_rows: query_copy's).
+bool chunk_direct(const ParamCtx &c, int layout, uint32_t digit_rows, uint32_t B, uint32_t kc) {
+  return (layout == PIR_LAYOUT_TENSOR || digit_rows) && query_ntt_fuses(c, B, kc);
+}
+// The query scratch of an answer in chunks of Kc ciphertexts: the copy in the GEMM's layout and
+// the NTT-form queries of the largest chunk whose NTT does not write that copy itself.
+struct QueryScratch {
+  size_t qhat_bytes;
+  QueryCopy copy;
+};
+QueryScratch query_scratch(const ParamCtx &c, int layout, uint32_t tile, uint32_t B, uint32_t D1, uint32_t D2,
+                           uint32_t Kc, bool tight) {
+  const uint64_t nslots = (uint64_t)c.p.L << c.logn;
+  QueryScratch q = {0, query_copy(layout, tile, nslots, Kc, 2 * B, D2, tight)};
+  for (uint32_t kc : {Kc, D1 % Kc})  // the last chunk may be shorter
+    if (!chunk_direct(c, layout, q.copy.rows, B, kc)) {
+      const size_t bytes = (size_t)B * kc * 2 * nslots * 4;
+      if (bytes > q.qhat_bytes) q.qhat_bytes = bytes;
+    }
+  return q;
 }
 uint32_t layout_tiles(int layout) {
   return layout == PIR_LAYOUT_PLAIN ? gemm_plain_tiles() : layout == PIR_LAYOUT_LIMB ? gemm_limb_tiles()
@@ -420,15 +456,13 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // GPU (a scratch allocation that then does not fit is refused with PIR_ERR_OOM,
     // after the cached memory has been given back).
     const size_t avail = available_device_bytes(db->device);
-    if (avail > 0) {
-      const size_t per_row = (size_t)B * 2 * L * n * 4 + layout_qs_bytes(db->layout, (uint64_t)L * n, 1, Mp);
-      const size_t budget = avail / 2;
-      if ((size_t)D1 * per_row > budget && per_row > 0) {
-        const size_t rows = budget / per_row;
-        const uint32_t chunks = (uint32_t)((D1 + (rows ? rows : 1) - 1) / (rows ? rows : 1));
-        Kc = (D1 + chunks - 1) / chunks;
-        if (Kc < kMinAutoChunk) Kc = kMinAutoChunk;
-      }
+    auto fits = [&](uint32_t kc) {
+      const QueryScratch q = query_scratch(c, db->layout, o.tile, B, D1, D2, plain ? kc : layout_chunk(db->layout, kc), false);
+      return q.qhat_bytes + q.copy.bytes <= avail / 2;
+    };
+    for (uint32_t chunks = 2; avail > 0 && Kc > kMinAutoChunk && !fits(Kc); ++chunks) {
+      Kc = (D1 + chunks - 1) / chunks;
+      if (Kc < kMinAutoChunk) Kc = kMinAutoChunk;
     }
   }
   if (!plain) {
@@ -461,10 +495,11 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     return PIR_ERR_ARG;
 
   // scratch: NTT'd query chunk | slot-major query chunk | slot-major results
-  const size_t qhat_bytes = qhat_ready ? 0 : (size_t)B * Kc * 2 * L * n * 4;
   // (the stall test hook belongs to the TMA scan)
   const uint32_t qtile = stall ? 7 : o.tile;
-  QueryCopy qc = query_copy(db->layout, qtile, nslots, Kc, M, D2, false);
+  QueryScratch qy = query_scratch(c, db->layout, qtile, B, D1, D2, Kc, false);
+  QueryScratch qt = query_scratch(c, db->layout, qtile, B, D1, D2, Kc, true);
+  if (qhat_ready) qy.qhat_bytes = qt.qhat_bytes = 0;
   const size_t out_bytes = nslots * M * D2 * 4;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   // Batch 1 on the TMA scan: the forward NTT writes the slot layout itself (pairs of
@@ -480,15 +515,13 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   // K-chunked fused path: the chunks before the last accumulate slot-major here
   const size_t slot_bytes = (fused && Kc < D1) ? out_bytes : 0;
   Scratch scratch(s);
-  const size_t other_bytes = up(qhat_bytes) + up(out_bytes) + up(full_bytes) + up(slot_bytes);
-  cudaError_t ae = scratch.alloc(other_bytes + up(qc.bytes));
-  if (ae == cudaErrorMemoryAllocation && qc.rows) {
-    cudaGetLastError();
-    qc = query_copy(db->layout, qtile, nslots, Kc, M, D2, true);
-    ae = scratch.alloc(other_bytes + up(qc.bytes));
-  }
-  CK(ae);
-  const size_t qs_bytes = qc.bytes;
+  const size_t other_bytes = up(out_bytes) + up(full_bytes) + up(slot_bytes);
+  bool took_tight = false;
+  CK(scratch.alloc_either(other_bytes + up(qy.qhat_bytes) + up(qy.copy.bytes),
+                          other_bytes + up(qt.qhat_bytes) + up(qt.copy.bytes), &took_tight));
+  if (took_tight) qy = qt;
+  const QueryCopy qc = qy.copy;
+  const size_t qhat_bytes = qy.qhat_bytes, qs_bytes = qc.bytes;
   char *base = static_cast<char *>(scratch.ptr);
   const uint32_t *qhat = qhat_ready ? qhat_ready : reinterpret_cast<uint32_t *>(base);
   void *qs = base + up(qhat_bytes);
@@ -544,8 +577,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // forward NTT of ciphertexts i0 .. i0+kc-1 of every query: per query b the rows
     // (b*D1 + i0)*2L .. +kc*2L are contiguous.
     const uint64_t G = (uint64_t)kc * 2 * L, S = (uint64_t)D1 * 2 * L;
-    const bool digits = db->layout == PIR_LAYOUT_TENSOR || qc.rows;
-    const bool direct = !qhat_ready && digits && query_ntt_fuses(c, B, kc);
+    const bool direct = !qhat_ready && chunk_direct(c, db->layout, qc.rows, B, kc);
     if (!qhat_ready && !direct) {
       tm.begin();
       CK(launch_ntt_fwd_rows(c, queries, (uint64_t)i0 * 2 * L, G, S, const_cast<uint32_t *>(qhat), (uint64_t)B * G,
@@ -698,15 +730,14 @@ pir_status_t session_open(pir_db *db, uint32_t B, uint32_t kc_max, cudaStream_t 
   ses->failed = PIR_OK;
   ses->qhat_bytes = (size_t)B * kc_max * ct * 4;
   QueryCopy qc = query_copy(db->layout, o.tile, nslots, kc_max, M, p.D2, false);
+  const QueryCopy qt = query_copy(db->layout, o.tile, nslots, kc_max, M, p.D2, true);
   ses->stage_bytes = up(ses->qhat_bytes);
   const size_t out_bytes = nslots * M * p.D2 * 4;
   void *mem = nullptr;
-  cudaError_t e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
-  if (e == cudaErrorMemoryAllocation && qc.rows) {
-    cudaGetLastError();
-    qc = query_copy(db->layout, o.tile, nslots, kc_max, M, p.D2, true);
-    e = malloc_async_retry(&mem, up(ses->qhat_bytes) + up(qc.bytes) + up(out_bytes), s);
-  }
+  const size_t other_bytes = up(ses->qhat_bytes) + up(out_bytes);
+  bool took_tight = false;
+  cudaError_t e = malloc_async_either(&mem, other_bytes + up(qc.bytes), other_bytes + up(qt.bytes), s, &took_tight);
+  if (took_tight) qc = qt;
   ses->qs_bytes = qc.bytes;
   ses->digit_rows = qc.rows;
   if (e == cudaSuccess) ses->mem = mem;
