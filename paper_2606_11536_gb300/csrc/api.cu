@@ -184,11 +184,13 @@ cudaError_t malloc_async_retry(void **ptr, size_t bytes, cudaStream_t s) {
 }
 
 // `bytes`, or where the device has no room for them the fewer `tight` (whether it was those:
-// *took_tight).
+// *took_tight).  The cached memory, which other streams may be about to use again, is given back
+// only where those do not fit either.
 cudaError_t malloc_async_either(void **ptr, size_t bytes, size_t tight, cudaStream_t s, bool *took_tight) {
   *took_tight = false;
-  const cudaError_t e = malloc_async_retry(ptr, bytes, s);
-  if (e != cudaErrorMemoryAllocation || tight >= bytes) return e;
+  if (tight >= bytes) return malloc_async_retry(ptr, bytes, s);
+  const cudaError_t e = cudaMallocAsync(ptr, bytes, s);
+  if (e != cudaErrorMemoryAllocation) return e;
   cudaGetLastError();
   *took_tight = true;
   return malloc_async_retry(ptr, tight, s);
