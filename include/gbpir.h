@@ -134,9 +134,9 @@ typedef struct {
                         this many ciphertexts (bounds the scratch to one chunk)     */
   uint32_t tile;     /* 0 = built-in choice; else a GEMM tile id (pir_gemm_tiles) that
                         holds the batch: plain 1, 2, 3 and 7 take at most 2, 4, 8 and
-                        8 query rows (2B), 7 also D2 <= 512, 9 (the tensor-core GEMM,
-                        the built-in choice for K-chunks of 128 rows and more) at
-                        least 3; limb 2 and 3 need the
+                        8 query rows (2B), 7 also D2 <= 512, 9 (the tensor-core GEMM)
+                        at least 3, 10 (the direct scan) D2 <= 512; pir_gemm_choice
+                        tells which is the built-in choice; limb 2 and 3 need the
                         rows padded to 16 to be multiples of 32 and 64 (limb 4, the
                         f16 tensor-core GEMM, is the built-in choice); tensor 1 is
                         the 1-SM GEMM, 2 the CTA-pair (2-SM) GEMM, which needs
@@ -425,6 +425,12 @@ const char *pir_last_cuda_error(void);
 
 /* Number of GEMM tile choices for a layout (ids 1..count for pir_answer_opts_t.tile). */
 uint32_t pir_gemm_tiles(int layout);
+
+/* The kernel that tile 0 stands for in an answer of B queries on a D1 x D2 database of this
+ * layout, as a tile id (10 wherever the plain layout's scan is the direct one, 7 where it is
+ * staged), on a device whose driver offers tensor maps.  With K-chunks, D1 is the chunk's rows.
+ * Host arithmetic only.  Errors: PIR_ERR_ARG (NULL, unknown layout, zero sizes). */
+pir_status_t pir_gemm_choice(int layout, uint32_t D1, uint32_t D2, uint32_t B, uint32_t *tile);
 
 /* Per-stage device time of the answers issued with PIR_ANSWER_STAGE_TIMES by the
  * calling thread since the last reset: waits for their events, adds each stage's

@@ -85,6 +85,7 @@ def lib():
             "pir_status_str": (C.c_char_p, [i32]),
             "pir_last_cuda_error": (C.c_char_p, []),
             "pir_gemm_tiles": (u32, [i32]),
+            "pir_gemm_choice": (i32, [i32, u32, u32, u32, C.POINTER(u32)]),
             "pir_stage_times": (i32, [C.POINTER(C.c_double), C.POINTER(C.c_uint64)]),
             "pir_kernel_launches": (C.c_uint64, []),
             "pir_check_device": (i32, [vp]),
@@ -415,6 +416,13 @@ def pir_status_str(status: int) -> str:
 
 def pir_gemm_tiles(layout: int) -> int:
     return int(lib().pir_gemm_tiles(layout))
+
+
+def pir_gemm_choice(layout: int, D1: int, D2: int, B: int) -> int:
+    """The tile id of the kernel that tile 0 stands for (host arithmetic only)."""
+    v = C.c_uint32()
+    _check(lib().pir_gemm_choice(layout, D1, D2, B, C.byref(v)), "pir_gemm_choice")
+    return int(v.value)
 
 
 PIR_ANSWER_STAGE_TIMES = 1

@@ -866,6 +866,20 @@ pir_status_t pir_stage_times(double *ms, uint64_t *launches) {
 
 uint64_t pir_kernel_launches(void) { return g_launches.load(); }
 
+pir_status_t pir_gemm_choice(int layout, uint32_t D1, uint32_t D2, uint32_t B, uint32_t *tile) {
+  if (!tile || D1 == 0 || D2 == 0 || B == 0 || B > 0x3fffffffu) return PIR_ERR_ARG;
+  const uint32_t M = 2 * B;
+  switch (layout) {
+    case PIR_LAYOUT_PLAIN:
+      *tile = gemm_plain_digits(M, D2, D1) ? kDigitTile : gemm_plain_core_choice(M, D2, D1);
+      if (*tile == 7 && !scan_staged_wins(M, D2, D1)) *tile = kDirectTile;
+      return PIR_OK;
+    case PIR_LAYOUT_LIMB: *tile = kLimbDigitTile; return PIR_OK;
+    case PIR_LAYOUT_TENSOR: *tile = gemm_tc_tile_ok(5, layout_rows(layout, M), D2) ? 5 : 1; return PIR_OK;
+  }
+  return PIR_ERR_ARG;
+}
+
 pir_status_t pir_release_memory(void) {
   release_cached_memory();
   return cuda_status(cudaGetLastError());
@@ -1494,17 +1508,16 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
   const pir_params_t &p = db->p;
   const uint32_t M = 2 * B, Mp16 = (M + 15u) & ~15u;
   const bool limb = db->layout == PIR_LAYOUT_LIMB;
-  std::vector<uint32_t> tiles;
+  std::vector<uint32_t> tiles;  // the built-in choice first: it wins ties
   if (db->layout == PIR_LAYOUT_TENSOR) {
-    for (uint32_t t : {1u, 2u, 5u})  // (3 and 4 are form 1)
+    for (uint32_t t : {5u, 1u, 2u})  // (3 and 4 are form 1)
       if (gemm_tc_tile_ok(t, layout_rows(db->layout, M), p.D2)) tiles.push_back(t);
   } else if (!limb) {
-    if (M <= 2) tiles.push_back(1);
-    if (M <= 4) tiles.push_back(2);
-    if (M <= 8) tiles.push_back(3);
-    if (gemm_plain_tile_ok(kDigitTile, M, p.D2)) tiles.push_back(kDigitTile);
-    for (uint32_t t = 4; t <= 6; ++t) tiles.push_back(t);
-    if (scan_tma_supports(M, p.D2)) tiles.push_back(7);
+    uint32_t first = gemm_uses_digits(db->layout, 0, M, p.D2, p.D1) ? kDigitTile : gemm_plain_core_choice(M, p.D2, p.D1);
+    if (first == kDirectTile && gemm_plain_tile_ok(7, M, p.D2)) first = 7;  // the same scan
+    tiles.push_back(first);
+    for (uint32_t t : {1u, 2u, 3u, kDigitTile, 4u, 5u, 6u, 7u, 8u})
+      if (t != first && gemm_plain_tile_ok(t, M, p.D2)) tiles.push_back(t);
   } else {
     if (gemm_limb_tile_ok(kLimbDigitTile, Mp16)) tiles.push_back(kLimbDigitTile);
     tiles.push_back(1);

@@ -185,6 +185,7 @@ cudaError_t launch_lwe_tc(const int8_t *A, uint32_t D1, uint32_t D0, const uint3
 // launch_query_digits from ciphertexts k0 .. k0 + Kc - 1 of qhat [B][Ks][2][L][n]; Mp a
 // multiple of 4 (on either layout), Kc <= kDigitMaxRows.
 constexpr uint32_t kDigitTile = 9, kLimbDigitTile = 4;
+constexpr uint32_t kDirectTile = 10;  // plain layout: the direct scan (scan_tma.cu)
 constexpr uint32_t kDigitMaxRows = 8192;
 bool gemm_digit_available();
 size_t gemm_digit_query_bytes(uint64_t nslots, uint32_t Kc, uint32_t Mp);
@@ -199,6 +200,7 @@ uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight);
 // Whether a layout's tile choice for chunks of Kc rows is the digit GEMM.
 bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc);
 bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc);  // gemm_plain.cu: tile 0's choice
+uint32_t gemm_plain_core_choice(uint32_t M, uint32_t D2, uint32_t Kc);  // and where that is not the digit GEMM
 
 // query_ntt.cu: ciphertexts i0 .. i0 + Kc - 1 of every query (queries [B][D1][2][L][n], coefficient
 // form) to the digits that launch_query_digits (plain, limb) or launch_query_to_tensor make of
@@ -211,6 +213,7 @@ cudaError_t launch_ntt_query_digits(const ParamCtx &c, int layout, const uint32_
 // TMA-staged stream; stall_test makes its consumers wait on a barrier that never
 // completes (exercises the bounded-wait error path).
 bool scan_tma_supports(uint32_t M, uint32_t D2);
+bool scan_staged_wins(uint32_t M, uint32_t D2, uint32_t Kc);  // which scan tile 7 is
 // out_poly = 1 writes the response layout [B][D2][2][L][n] (NTT domain) directly.
 // acc_src, when set, is a slot-major partial result [L*n][M][D2] added in before the
 // write (the K-chunks before the last accumulate there with coalesced accesses).

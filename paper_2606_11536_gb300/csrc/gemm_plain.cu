@@ -351,8 +351,9 @@ bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc) {
 // (one query row per thread, for a few queries).  Where the digit GEMM does not apply, 0
 // picks the TMA scan up to 4 rows, the 8-row GEMM up to 8, else a GEMM tile by M.
 // 9 = the tensor-core GEMM over in-kernel digits (gemm_digit.cu), which takes another
-// query operand and is launched by its own entry point.
-uint32_t gemm_plain_tiles() { return kDigitTile; }
+// query operand and is launched by its own entry point.  10 = the direct scan for any number of
+// rows (D2 <= 512).
+uint32_t gemm_plain_tiles() { return kDirectTile; }
 
 bool gemm_plain_tile_ok(uint32_t tile, uint32_t M, uint32_t D2) {
   switch (tile) {
@@ -362,27 +363,25 @@ bool gemm_plain_tile_ok(uint32_t tile, uint32_t M, uint32_t D2) {
     case 2: return M <= 4;
     case 3: return M <= 8;
     case 7: return scan_tma_supports(M, D2);
+    case kDirectTile: return D2 <= kScanCols;
   }
   return false;
+}
+
+// What tile 0 runs on the CUDA cores: the scans up to 4 query rows; from 5 on the direct scan
+// against the GEMM tile that holds the rows (5-8 rows: the 8-row GEMM tile measured 15-17% ahead
+// of the GEMV)
+uint32_t gemm_plain_core_choice(uint32_t M, uint32_t D2, uint32_t Kc) {
+  const Costs t = costs(M, D2, Kc);
+  if (D2 <= kScanCols && M > 4 && t.direct < kMargin * t.core) return kDirectTile;
+  if (M <= 4 && scan_tma_supports(M, D2)) return 7;
+  return M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 8 : M <= 16 ? 4 : M <= 32 ? 5 : 6;
 }
 
 cudaError_t launch_gemm_plain(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
                               uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
                               uint32_t tile, int stall_test, cudaStream_t s) {
-  if (tile == 0) {
-    // the scans up to 4 query rows; from 5 on the direct scan against the GEMM tile that holds
-    // the rows (5-8 rows: the 8-row GEMM tile measured 15-17% ahead of the GEMV)
-    const Costs t = costs(M, D2, Kc);
-    if (D2 <= kScanCols && M > 4 && t.direct < kMargin * t.core)
-      return launch_scan_direct(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, 0, nullptr, s);
-    if (M <= 4 && scan_tma_supports(M, D2)) tile = 7;
-    else if (M <= 2) tile = 1;
-    else if (M <= 4) tile = 2;
-    else if (M <= 8) tile = 8;
-    else if (M <= 16) tile = 4;
-    else if (M <= 32) tile = 5;
-    else tile = 6;
-  }
+  if (tile == 0) tile = gemm_plain_core_choice(M, D2, Kc);
   if (stall_test && tile != 7) return cudaErrorInvalidValue;
   switch (tile) {
     case 7: return launch_scan_tma(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, stall_test, 0, nullptr, s);
@@ -398,6 +397,9 @@ cudaError_t launch_gemm_plain(const ParamCtx &c, const uint32_t *db, uint32_t D1
     // 3.4% faster at 2B = 64; 32-row stages
     case 6: return gemm_launch<64, 128, 8, 32, 128, 3>(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, s);
     case 8: return gemm_launch<8, 256, 1>(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, s);
+    case kDirectTile:
+      return D2 <= kScanCols ? launch_scan_direct(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, 0, nullptr, s)
+                             : cudaErrorInvalidValue;
   }
   return cudaErrorInvalidValue;
 }

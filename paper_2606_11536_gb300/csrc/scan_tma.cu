@@ -399,18 +399,16 @@ cudaError_t scan_launch(const ParamCtx &c, const ScanArgs &a0, cudaStream_t s) {
 
 }  // namespace
 
-namespace {
 // Whether the staged stream is the faster scan.  It is where a row fills its eight warps' quads
 // (one or two each) and a slot is long enough; one query: 64 x 256 112 against 123 us direct,
 // 512 x 256 654 against 797, 256 x 460 629 against 818; but 16 x 256 58 against 45, 32 x 512 135
 // against 122, 256 x 160 (by rate) and 256 x 400 847 against 672.  Two queries: 512 x 256 1060
 // against 1127, 512 x 512 3040 against 2136, 64 x 256 188 against 164.  Four: always slower.
-bool staged_wins(uint32_t M, uint32_t D2, uint32_t Kc) {
+bool scan_staged_wins(uint32_t M, uint32_t D2, uint32_t Kc) {
   const uint64_t bytes = (uint64_t)Kc * D2 * 4;
   if (D2 <= 256) return D2 >= 192 && (M <= 2 ? bytes >= (64u << 10) : M <= 4 && bytes >= (128u << 10));
   return D2 >= 448 && M <= 2 && bytes >= (128u << 10);
 }
-}  // namespace
 
 cudaError_t launch_scan_direct(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
                                uint32_t M, uint32_t Mp, uint32_t i0, uint32_t Kc, uint32_t *out, int acc,
@@ -443,7 +441,7 @@ cudaError_t launch_scan_tma(const ParamCtx &c, const uint32_t *db, uint32_t D1, 
   // query rows are bulk-copied: Mp = 2 needs an even Kc (16-byte chunk starts)
   if (!scan_tma_supports(M, D2) || Kc == 0 || !(Mp % 4 == 0 || (Mp == 2 && M <= 2 && Kc % 2 == 0)))
     return cudaErrorInvalidValue;
-  if (!stall_test && !staged_wins(M, D2, Kc))
+  if (!stall_test && !scan_staged_wins(M, D2, Kc))
     return launch_scan_direct(c, db, D1, D2, qs, M, Mp, i0, Kc, out, acc, out_poly, acc_src, s);
   uint32_t *err = nullptr;
   cudaError_t e = device_error_word(&err);
