@@ -360,13 +360,14 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     M = 2 * B
     nslots = L_PRIMES * n
     launch_ms = gemm_ms / launches_per_step
-    # the digit GEMM: its tile ids, or the default tile (plain: from two queries and 128 rows on)
-    digits = ((layout == g.PIR_LAYOUT_PLAIN and (tile == 9 or (tile == 0 and M >= 3 and D1 >= 128)))
-              or (layout == g.PIR_LAYOUT_LIMB and tile in (0, 4)))
-    streaming = (layout == g.PIR_LAYOUT_PLAIN and not digits and M <= 8
-                 and (tile in (1, 2, 3, 7) or (tile == 0 and M <= 4 and D2 <= 512)))
+    rows = -(-D1 // launches_per_step)  # of one launch
+    choice = g.pir_gemm_choice(layout, rows, D2, B)
+    # the kernel that ran, as a tile id (tile 7 is the staged or, 10, the direct scan)
+    ran = choice if tile == 0 or (layout == g.PIR_LAYOUT_PLAIN and tile == 7 and choice == 10) else tile
+    digits = (layout, ran) in ((g.PIR_LAYOUT_PLAIN, 9), (g.PIR_LAYOUT_LIMB, 4))
+    streaming = layout == g.PIR_LAYOUT_PLAIN and M <= 8 and ran in (1, 2, 3, 7, 10)
     if streaming:
-        kernel_tag = "scan_tma" if tile in (0, 7) else "gemv_scan"
+        kernel_tag = {7: "scan_tma", 10: "scan_direct"}.get(ran, "gemv_scan")
         alg_bytes = nslots * (D1 * D2 * 4 + D1 * M * 4 + M * D2 * 4)
         per = alg_bytes / launches_per_step
         rl = {"bound": "hbm", "achieved": per / (launch_ms / 1e3) / 1e9, "peak": float(ctx.peaks["hbm_gbs"]),
@@ -414,7 +415,7 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     rl["launches_per_step"] = launches_per_step
     rl["alg_bytes_per_launch"] = per
     src = os.path.join(ROOT, "paper_2606_11536_gb300", "csrc",
-                       {"scan_tma": "scan_tma.cu", "gemv_scan": "gemm_plain.cu", "gemm_plain": "gemm_plain.cu",
+                       {"scan_tma": "scan_tma.cu", "scan_direct": "scan_tma.cu", "gemv_scan": "gemm_plain.cu", "gemm_plain": "gemm_plain.cu",
                         "gemm_limb": "gemm_limb.cu", "gemm_tc": "gemm_tc.cu", "gemm_digit": "gemm_digit.cu",
                         "gemm_digit_limb": "gemm_digit.cu"}[kernel_tag])
     rl["traffic"] = profile_traffic(kernel_tag, ctx.wl, B, src, launches_per_step)
