@@ -432,6 +432,13 @@ uint32_t pir_gemm_tiles(int layout);
  * Host arithmetic only.  Errors: PIR_ERR_ARG (NULL, unknown layout, zero sizes). */
 pir_status_t pir_gemm_choice(int layout, uint32_t D1, uint32_t D2, uint32_t B, uint32_t *tile);
 
+/* Device scratch of one pir_answer of B queries where memory is plentiful (all of D1 at once, or
+ * in the layout's largest chunks), on a device whose driver offers tensor maps: the queries in
+ * the GEMM's layout, their NTT-form copy where one is made, and the slot-major result.  n, L, D1
+ * and D2 of params count.  Host arithmetic only.  Errors: PIR_ERR_ARG (NULL, unknown layout, zero
+ * sizes). */
+pir_status_t pir_answer_scratch_bytes(const pir_params_t *params, int layout, uint32_t B, size_t *bytes);
+
 /* Per-stage device time of the answers issued with PIR_ANSWER_STAGE_TIMES by the
  * calling thread since the last reset: waits for their events, adds each stage's
  * elapsed milliseconds into ms[PIR_STAGES] and its kernel launches into

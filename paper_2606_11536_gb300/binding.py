@@ -86,6 +86,7 @@ def lib():
             "pir_last_cuda_error": (C.c_char_p, []),
             "pir_gemm_tiles": (u32, [i32]),
             "pir_gemm_choice": (i32, [i32, u32, u32, u32, C.POINTER(u32)]),
+            "pir_answer_scratch_bytes": (i32, [P, i32, u32, C.POINTER(sz)]),
             "pir_stage_times": (i32, [C.POINTER(C.c_double), C.POINTER(C.c_uint64)]),
             "pir_kernel_launches": (C.c_uint64, []),
             "pir_check_device": (i32, [vp]),
@@ -583,13 +584,19 @@ def raw_db_bytes(p) -> int:
 
 
 def answer_scratch_bytes(p, layout: int, B: int) -> int:
-    """Device scratch one answer of B queries takes inside the library with the whole
-    of D1 at once: the NTT-form query copy (4 bytes per residue), the queries in the
-    GEMM's layout (4 bytes per residue; 8 for the tensor layout's bf16 digits) and
-    the slot-major result (4 bytes per residue of the 2B x D2 result polynomials)."""
+    """Device scratch to set aside for one answer of B queries: per query the NTT-form copy
+    (4 bytes per residue), the queries in the GEMM's layout (4 bytes per residue; 8 for the
+    tensor layout's bf16 digits) and the slot-major result (4 bytes per residue of the 2B x D2
+    result polynomials); or what the library says that it takes, where its digits (8 bytes per
+    residue of padded rows) come to more: small batches, which keep both copies."""
     per_q = 2 * p.L * p.n * 4  # one ciphertext
     layout_q = 2 if layout == PIR_LAYOUT_TENSOR else 1
-    return B * (p.D1 * per_q * (1 + layout_q) + p.D2 * per_q)
+    flat = B * (p.D1 * per_q * (1 + layout_q) + p.D2 * per_q)
+    if layout == PIR_LAYOUT_PLAIN and pir_gemm_choice(layout, p.D1, p.D2, B) != 9:
+        return flat
+    q, v = pir_params_t(n=p.n, L=p.L, D1=p.D1, D2=p.D2), C.c_size_t()
+    _check(lib().pir_answer_scratch_bytes(C.byref(q), layout, B, C.byref(v)), "pir_answer_scratch_bytes")
+    return max(flat, int(v.value))
 
 
 def resident_db_bytes(p, layout: int = PIR_LAYOUT_PLAIN) -> int:

@@ -250,19 +250,21 @@ struct QueryCopy {
   size_t bytes;
   uint32_t rows;
 };
-QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t D2, bool tight) {
+QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t D2, bool tight,
+                     bool maps = gemm_digit_available()) {
   const size_t b = layout_qs_bytes(layout, nslots, Kc, layout_rows(layout, M));
-  if (!gemm_uses_digits(layout, tile, M, D2, Kc)) return {b, 0};
+  if (!gemm_uses_digits(layout, tile, M, D2, Kc, maps)) return {b, 0};
   // fewer than 128 plain rows: digits (of 64 rows at least) take more than the tiles' copy
   if (tight && layout == PIR_LAYOUT_PLAIN && tile == 0 && Kc < 128) return {b, 0};
   const uint32_t rows = gemm_digit_rows(nslots, Kc, round4(M), tight);
   const size_t d = gemm_digit_query_bytes(nslots, rows, round4(M));
-  return {d > b ? d : b, rows};
+  // (the last chunk's piece of a plain database may take the tiles' copy)
+  return {layout == PIR_LAYOUT_LIMB || d > b ? d : b, rows};
 }
 // Whether the forward NTT of a chunk of kc ciphertexts writes the GEMM's digits itself
 // (digit_rows: query_copy's).
-bool chunk_direct(const ParamCtx &c, int layout, uint32_t digit_rows, uint32_t B, uint32_t kc) {
-  return (layout == PIR_LAYOUT_TENSOR || digit_rows) && query_ntt_fuses(c, B, kc);
+bool chunk_direct(uint32_t L, int layout, uint32_t digit_rows, uint32_t B, uint32_t kc) {
+  return (layout == PIR_LAYOUT_TENSOR || digit_rows) && query_ntt_fuses(L, B, kc);
 }
 // The query scratch of an answer in chunks of Kc ciphertexts: the copy in the GEMM's layout and
 // the NTT-form queries of the largest chunk whose NTT does not write that copy itself.
@@ -270,12 +272,12 @@ struct QueryScratch {
   size_t qhat_bytes;
   QueryCopy copy;
 };
-QueryScratch query_scratch(const ParamCtx &c, int layout, uint32_t tile, uint32_t B, uint32_t D1, uint32_t D2,
-                           uint32_t Kc, bool tight) {
-  const uint64_t nslots = (uint64_t)c.p.L << c.logn;
-  QueryScratch q = {0, query_copy(layout, tile, nslots, Kc, 2 * B, D2, tight)};
+QueryScratch query_scratch(uint32_t n, uint32_t L, int layout, uint32_t tile, uint32_t B, uint32_t D1, uint32_t D2,
+                           uint32_t Kc, bool tight, bool maps = gemm_digit_available()) {
+  const uint64_t nslots = (uint64_t)L * n;
+  QueryScratch q = {0, query_copy(layout, tile, nslots, Kc, 2 * B, D2, tight, maps)};
   for (uint32_t kc : {Kc, D1 % Kc})  // the last chunk may be shorter
-    if (!chunk_direct(c, layout, q.copy.rows, B, kc)) {
+    if (!chunk_direct(L, layout, q.copy.rows, B, kc)) {
       const size_t bytes = (size_t)B * kc * 2 * nslots * 4;
       if (bytes > q.qhat_bytes) q.qhat_bytes = bytes;
     }
@@ -459,7 +461,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // after the cached memory has been given back).
     const size_t avail = available_device_bytes(db->device);
     auto fits = [&](uint32_t kc) {
-      const QueryScratch q = query_scratch(c, db->layout, o.tile, B, D1, D2, plain ? kc : layout_chunk(db->layout, kc), false);
+      const QueryScratch q = query_scratch(n, L, db->layout, o.tile, B, D1, D2, plain ? kc : layout_chunk(db->layout, kc), false);
       return q.qhat_bytes + q.copy.bytes <= avail / 2;
     };
     for (uint32_t chunks = 2; avail > 0 && Kc > kMinAutoChunk && !fits(Kc); ++chunks) {
@@ -499,8 +501,8 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   // scratch: NTT'd query chunk | slot-major query chunk | slot-major results
   // (the stall test hook belongs to the TMA scan)
   const uint32_t qtile = stall ? 7 : o.tile;
-  QueryScratch qy = query_scratch(c, db->layout, qtile, B, D1, D2, Kc, false);
-  QueryScratch qt = query_scratch(c, db->layout, qtile, B, D1, D2, Kc, true);
+  QueryScratch qy = query_scratch(n, L, db->layout, qtile, B, D1, D2, Kc, false);
+  QueryScratch qt = query_scratch(n, L, db->layout, qtile, B, D1, D2, Kc, true);
   if (qhat_ready) qy.qhat_bytes = qt.qhat_bytes = 0;
   const size_t out_bytes = nslots * M * D2 * 4;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -510,6 +512,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
   // (every chunk, the last included, must hold an even number of ciphertexts)
   const bool fused = !qhat_ready && plain && B == 1 && (o.tile == 0 || o.tile == 7) && scan_tma_supports(M, D2) &&
                      Kc % 2 == 0 && D1 % 2 == 0;
+  if (fused) qy.copy = qt.copy = {0, 0};
   // full-modulus responses before switching: the unused result area on the fused
   // path (the same size at B = 1), an area of their own otherwise
   StageTimer tm((o.flags & PIR_ANSWER_STAGE_TIMES) != 0, s);
@@ -579,7 +582,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // forward NTT of ciphertexts i0 .. i0+kc-1 of every query: per query b the rows
     // (b*D1 + i0)*2L .. +kc*2L are contiguous.
     const uint64_t G = (uint64_t)kc * 2 * L, S = (uint64_t)D1 * 2 * L;
-    const bool direct = !qhat_ready && chunk_direct(c, db->layout, qc.rows, B, kc);
+    const bool direct = !qhat_ready && chunk_direct(L, db->layout, qc.rows, B, kc);
     if (!qhat_ready && !direct) {
       tm.begin();
       CK(launch_ntt_fwd_rows(c, queries, (uint64_t)i0 * 2 * L, G, S, const_cast<uint32_t *>(qhat), (uint64_t)B * G,
@@ -878,6 +881,17 @@ pir_status_t pir_gemm_choice(int layout, uint32_t D1, uint32_t D2, uint32_t B, u
     case PIR_LAYOUT_TENSOR: *tile = gemm_tc_tile_ok(5, layout_rows(layout, M), D2) ? 5 : 1; return PIR_OK;
   }
   return PIR_ERR_ARG;
+}
+
+pir_status_t pir_answer_scratch_bytes(const pir_params_t *params, int layout, uint32_t B, size_t *bytes) {
+  if (!params || !bytes || B == 0 || B > 0x3fffffffu || params->D1 == 0 || params->D2 == 0) return PIR_ERR_ARG;
+  if (layout < PIR_LAYOUT_PLAIN || layout > PIR_LAYOUT_TENSOR) return PIR_ERR_ARG;
+  const pir_params_t &p = *params;
+  const uint32_t Kc = layout == PIR_LAYOUT_PLAIN ? p.D1 : layout_chunk(layout, p.D1);
+  const QueryScratch q = query_scratch(p.n, p.L, layout, 0, B, p.D1, p.D2, Kc, false, true);
+  const bool fused = layout == PIR_LAYOUT_PLAIN && B == 1 && scan_tma_supports(2, p.D2) && p.D1 % 2 == 0;
+  *bytes = q.qhat_bytes + (fused ? 0 : q.copy.bytes) + (size_t)p.L * p.n * 2 * B * p.D2 * 4;
+  return PIR_OK;
 }
 
 pir_status_t pir_release_memory(void) {
@@ -1513,7 +1527,7 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
     for (uint32_t t : {5u, 1u, 2u})  // (3 and 4 are form 1)
       if (gemm_tc_tile_ok(t, layout_rows(db->layout, M), p.D2)) tiles.push_back(t);
   } else if (!limb) {
-    uint32_t first = gemm_uses_digits(db->layout, 0, M, p.D2, p.D1) ? kDigitTile : gemm_plain_core_choice(M, p.D2, p.D1);
+    uint32_t first = gemm_uses_digits(db->layout, 0, M, p.D2, p.D1, gemm_digit_available()) ? kDigitTile : gemm_plain_core_choice(M, p.D2, p.D1);
     if (first == kDirectTile && gemm_plain_tile_ok(7, M, p.D2)) first = 7;  // the same scan
     tiles.push_back(first);
     for (uint32_t t : {1u, 2u, 3u, kDigitTile, 4u, 5u, 6u, 7u, 8u})

@@ -174,7 +174,7 @@ cudaError_t query_layout(int layout, const QueryArgs &a, uint32_t Uc, cudaStream
 
 // Eight rows a CTA fill the SMs twice from 4096 rows on (5418: 134 -> 101 us); below, a transform
 // of one row a CTA and the transpose are the shorter chain.
-bool query_ntt_fuses(const ParamCtx &c, uint32_t B, uint32_t Kc) { return (uint64_t)B * Kc * 2 * c.p.L >= 4096; }
+bool query_ntt_fuses(uint32_t L, uint32_t B, uint32_t Kc) { return (uint64_t)B * Kc * 2 * L >= 4096; }
 
 cudaError_t launch_ntt_query_digits(const ParamCtx &c, int layout, const uint32_t *queries, uint32_t B, uint32_t D1,
                                     uint32_t i0, uint32_t Kc, uint32_t Mp, uint16_t *qt, cudaStream_t s) {

@@ -277,16 +277,15 @@ class Server:
             q = self.queues[name]
             info = self.dbs[name]
             p = info["params"]
-            # one request's device memory while its batch runs: its query and response
-            # buffers and the answer's own scratch (NTT-form copy, GEMM layout, result)
-            per_query = 8 * p.L * p.n * (p.D1 + p.D2) + binding.answer_scratch_bytes(p, info.get("layout", 0), 1)
             nb = min(self.max_batch, _per_db(self.db_max_batch, name, self.max_batch), len(q))
             if self.scratch_budget is not None:
-                nb = min(nb, (self.scratch_budget - self.scratch_in_flight) // per_query)
-                if nb <= 0:
-                    if self.scratch_in_flight:
-                        break  # wait for batches in flight to release memory
-                    nb = 1  # a single request larger than the budget still runs, alone
+                left = self.scratch_budget - self.scratch_in_flight
+                while nb > 1 and self._batch_bytes(info, nb) > left:
+                    nb -= 1
+                # wait for batches in flight to release memory; a single request larger
+                # than the budget still runs, alone
+                if self._batch_bytes(info, nb) > left and self.scratch_in_flight:
+                    break
             take = [q.popleft() for _ in range(nb)]
             t = self.clock()
             for r in take:
@@ -301,10 +300,21 @@ class Server:
                     r.status = e.status
                     self.failed.append(r)
                 continue
-            s.busy, s.requests, s.db, s.scratch, s.t_dispatch = True, take, name, nb * per_query, t
+            s.busy, s.requests, s.db, s.t_dispatch = True, take, name, t
+            s.scratch = self._batch_bytes(info, nb) if self.scratch_budget is not None else 0
             self.scratch_in_flight += s.scratch
         self.done.extend(finished)
         return finished
+
+    @staticmethod
+    def _batch_bytes(info, nb) -> int:
+        """Device memory of a batch while it runs: its query and response buffers and the
+        answer's own scratch (NTT-form copy, GEMM layout, result)."""
+        known = info.setdefault("batch_bytes", {})
+        if nb not in known:
+            p = info["params"]
+            known[nb] = nb * 8 * p.L * p.n * (p.D1 + p.D2) + binding.answer_scratch_bytes(p, info.get("layout", 0), nb)
+        return known[nb]
 
     def _next_db(self) -> Optional[str]:
         """The database whose oldest waiting request arrived first, among those
