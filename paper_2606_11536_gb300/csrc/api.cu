@@ -253,7 +253,7 @@ struct QueryCopy {
 QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, uint32_t M, uint32_t D2, bool tight,
                      bool maps = gemm_digit_available()) {
   const size_t b = layout_qs_bytes(layout, nslots, Kc, layout_rows(layout, M));
-  if (!gemm_uses_digits(layout, tile, M, D2, Kc, maps)) return {b, 0};
+  if (!gemm_uses_digits(layout, tile, M, D2, Kc, false, maps)) return {b, 0};
   // fewer than 128 plain rows: digits (of 64 rows at least) take more than the tiles' copy
   if (tight && layout == PIR_LAYOUT_PLAIN && tile == 0 && Kc < 128) return {b, 0};
   const uint32_t rows = gemm_digit_rows(nslots, Kc, round4(M), tight);
@@ -261,10 +261,16 @@ QueryCopy query_copy(int layout, uint32_t tile, uint64_t nslots, uint32_t Kc, ui
   // (the last chunk's piece of a plain database may take the tiles' copy)
   return {layout == PIR_LAYOUT_LIMB || d > b ? d : b, rows};
 }
-// Whether the forward NTT of a chunk of kc ciphertexts writes the GEMM's digits itself
-// (digit_rows: query_copy's).
-bool chunk_direct(uint32_t L, int layout, uint32_t digit_rows, uint32_t B, uint32_t kc) {
-  return (layout == PIR_LAYOUT_TENSOR || digit_rows) && query_ntt_fuses(L, B, kc);
+// Whether a chunk of kc ciphertexts runs on the digit GEMM (digit_rows: query_copy's for the
+// largest chunk; shorter ones, and those that add to earlier ones, choose for themselves), and
+// whether their forward NTT writes the GEMM's digits itself.
+bool chunk_digits(int layout, uint32_t tile, uint32_t digit_rows, uint32_t B, uint32_t D2, uint32_t kc, bool acc) {
+  return digit_rows && gemm_uses_digits(layout, tile, 2 * B, D2, kc, acc, true);
+}
+bool chunk_direct(uint32_t L, int layout, uint32_t tile, uint32_t digit_rows, uint32_t B, uint32_t D2, uint32_t kc,
+                  bool acc) {
+  return (layout == PIR_LAYOUT_TENSOR || chunk_digits(layout, tile, digit_rows, B, D2, kc, acc)) &&
+         query_ntt_fuses(L, B, kc);
 }
 // The query scratch of an answer in chunks of Kc ciphertexts: the copy in the GEMM's layout and
 // the NTT-form queries of the largest chunk whose NTT does not write that copy itself.
@@ -276,11 +282,14 @@ QueryScratch query_scratch(uint32_t n, uint32_t L, int layout, uint32_t tile, ui
                            uint32_t Kc, bool tight, bool maps = gemm_digit_available()) {
   const uint64_t nslots = (uint64_t)L * n;
   QueryScratch q = {0, query_copy(layout, tile, nslots, Kc, 2 * B, D2, tight, maps)};
-  for (uint32_t kc : {Kc, D1 % Kc})  // the last chunk may be shorter
-    if (!chunk_direct(L, layout, q.copy.rows, B, kc)) {
-      const size_t bytes = (size_t)B * kc * 2 * nslots * 4;
-      if (bytes > q.qhat_bytes) q.qhat_bytes = bytes;
-    }
+  auto chunk = [&](uint32_t kc, bool acc) {
+    if (kc == 0 || chunk_direct(L, layout, tile, q.copy.rows, B, D2, kc, acc)) return;
+    const size_t bytes = (size_t)B * kc * 2 * nslots * 4;
+    if (bytes > q.qhat_bytes) q.qhat_bytes = bytes;
+  };
+  chunk(Kc, false);
+  if (D1 / 2 >= Kc) chunk(Kc, true);
+  chunk(D1 % Kc, true);  // the last one may be shorter
   return q;
 }
 uint32_t layout_tiles(int layout) {
@@ -393,7 +402,7 @@ pir_status_t chunk_gemm(const pir_db *db, const uint32_t *qhat, uint32_t B, uint
                         cudaStream_t s, const uint32_t *queries = nullptr) {
   const ParamCtx &c = *db->ctx;
   const uint32_t D1 = db->p.D1, D2 = db->p.D2, M = 2 * B;
-  if (digit_rows) {
+  if (chunk_digits(db->layout, tile, digit_rows, B, D2, kc, i0 > 0)) {
     uint16_t *qt = static_cast<uint16_t *>(qs);
     for (uint32_t k0 = 0; k0 < kc; k0 += digit_rows) {
       const uint32_t kr = kc - k0 < digit_rows ? kc - k0 : digit_rows;
@@ -582,7 +591,7 @@ pir_status_t answer_device(pir_db *db, const uint32_t *queries, uint32_t B, uint
     // forward NTT of ciphertexts i0 .. i0+kc-1 of every query: per query b the rows
     // (b*D1 + i0)*2L .. +kc*2L are contiguous.
     const uint64_t G = (uint64_t)kc * 2 * L, S = (uint64_t)D1 * 2 * L;
-    const bool direct = !qhat_ready && chunk_direct(L, db->layout, qc.rows, B, kc);
+    const bool direct = !qhat_ready && chunk_direct(L, db->layout, o.tile, qc.rows, B, D2, kc, i0 > 0);
     if (!qhat_ready && !direct) {
       tm.begin();
       CK(launch_ntt_fwd_rows(c, queries, (uint64_t)i0 * 2 * L, G, S, const_cast<uint32_t *>(qhat), (uint64_t)B * G,
@@ -874,7 +883,7 @@ pir_status_t pir_gemm_choice(int layout, uint32_t D1, uint32_t D2, uint32_t B, u
   const uint32_t M = 2 * B;
   switch (layout) {
     case PIR_LAYOUT_PLAIN:
-      *tile = gemm_plain_digits(M, D2, D1) ? kDigitTile : gemm_plain_core_choice(M, D2, D1);
+      *tile = gemm_plain_digits(M, D2, D1, false) ? kDigitTile : gemm_plain_core_choice(M, D2, D1);
       if (*tile == 7 && !scan_staged_wins(M, D2, D1)) *tile = kDirectTile;
       return PIR_OK;
     case PIR_LAYOUT_LIMB: *tile = kLimbDigitTile; return PIR_OK;
@@ -1527,7 +1536,7 @@ pir_status_t pir_autotune(pir_db_t db, uint32_t B, void *stream, uint32_t reps, 
     for (uint32_t t : {5u, 1u, 2u})  // (3 and 4 are form 1)
       if (gemm_tc_tile_ok(t, layout_rows(db->layout, M), p.D2)) tiles.push_back(t);
   } else if (!limb) {
-    uint32_t first = gemm_uses_digits(db->layout, 0, M, p.D2, p.D1, gemm_digit_available()) ? kDigitTile : gemm_plain_core_choice(M, p.D2, p.D1);
+    uint32_t first = gemm_uses_digits(db->layout, 0, M, p.D2, p.D1, false, gemm_digit_available()) ? kDigitTile : gemm_plain_core_choice(M, p.D2, p.D1);
     if (first == kDirectTile && gemm_plain_tile_ok(7, M, p.D2)) first = 7;  // the same scan
     tiles.push_back(first);
     for (uint32_t t : {1u, 2u, 3u, kDigitTile, 4u, 5u, 6u, 7u, 8u})

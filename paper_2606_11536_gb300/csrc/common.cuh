@@ -197,10 +197,11 @@ cudaError_t launch_gemm_digit(const ParamCtx &c, int layout, const void *db, uin
 // Rows of one digit GEMM of a chunk of Kc rows.  Its query digits take 8 bytes per
 // residue where the other tiles' query copy takes 4.
 uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight);
-// Whether a layout's tile choice for chunks of Kc rows is the digit GEMM; maps: whether the driver
-// offers the tensor maps that it needs (gemm_digit_available).
-bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc, bool maps);
-bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc);  // gemm_plain.cu: tile 0's choice
+// Whether a layout's tile choice for a chunk of Kc rows is the digit GEMM.  acc: the chunk adds to
+// earlier ones; maps: whether the driver offers the tensor maps that it needs
+// (gemm_digit_available).
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc, bool acc, bool maps);
+bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc, bool acc);  // gemm_plain.cu: tile 0's choice
 uint32_t gemm_plain_core_choice(uint32_t M, uint32_t D2, uint32_t Kc);  // and where that is not the digit GEMM
 
 // query_ntt.cu: ciphertexts i0 .. i0 + Kc - 1 of every query (queries [B][D1][2][L][n], coefficient

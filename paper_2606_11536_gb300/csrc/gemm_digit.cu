@@ -626,14 +626,14 @@ uint32_t gemm_digit_rows(uint64_t nslots, uint32_t Kc, uint32_t Mp, bool tight) 
   return r < 64 ? 64 : r > kDigitMaxRows ? kDigitMaxRows : r;
 }
 
-bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc, bool maps) {
+bool gemm_uses_digits(int layout, uint32_t tile, uint32_t M, uint32_t D2, uint32_t Kc, bool acc, bool maps) {
   if (layout == PIR_LAYOUT_TENSOR) return false;
   if (tile == (layout == PIR_LAYOUT_PLAIN ? kDigitTile : kLimbDigitTile)) return true;
   if (tile != 0 || !maps) return false;
   // INT8 mma.sync at its peak is 1.3 to 7 times slower at every size measured (32 to 512 rows
   // and columns, 1 to 32 queries).
   if (layout == PIR_LAYOUT_LIMB) return true;
-  return gemm_plain_digits(M, D2, Kc);
+  return gemm_plain_digits(M, D2, Kc, acc);
 }
 
 bool gemm_digit_available() { return tensor_maps_available(); }

@@ -338,11 +338,15 @@ Costs costs(uint32_t M, uint32_t D2, uint32_t Kc) {
 }  // namespace
 
 // One query streams the DB at HBM speed on the CUDA cores already.  From 128 rows on the digit
-// GEMM wins at every width (1.2x at 512 columns and batch 4, up to 4x).
-bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc) {
+// GEMM wins at every width (1.2x at 512 columns and batch 4, up to 4x).  A chunk that adds to
+// earlier ones reads their sums: per 4096 slots that costs the digit GEMM up to 0.047 us for each
+// row and column (3 to 24 queries; 0.008 else), the others at most 0.005.  512 columns, 8 queries, us:
+// 16 rows 413, adding 763 (124 by the tile); 128 rows 418, 775 (625); 192 rows 514, 801 (913).
+bool gemm_plain_digits(uint32_t M, uint32_t D2, uint32_t Kc, bool acc) {
   if (M < 3) return false;
-  if (Kc >= 128) return true;
-  const Costs t = costs(M, D2, Kc);
+  if (Kc >= (acc ? 192 : 128)) return true;
+  Costs t = costs(M, D2, Kc);
+  if (acc) t.digit += (M > 4 && M <= 48 ? 0.044f : 0.008f) * (float)M * (float)D2;
   return (t.digit < t.direct || D2 > kScanCols) && (M <= 4 || t.digit < kMargin * t.core);
 }
 
