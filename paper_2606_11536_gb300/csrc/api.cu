@@ -40,6 +40,14 @@ std::atomic<uint64_t> g_launches{0};
 namespace {
 std::mutex g_err_mu;
 uint32_t *g_err_word[64] = {};
+__device__ uint32_t g_device_error;
+
+// Set-up that is not part of a stream's work, also where the calling thread captures a stream.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 }  // namespace
 
 cudaError_t device_error_word(uint32_t **word) {
@@ -49,11 +57,12 @@ cudaError_t device_error_word(uint32_t **word) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_err_mu);
   if (!g_err_word[dev]) {
-    uint32_t *w = nullptr;
-    if ((e = cudaMalloc(&w, sizeof(uint32_t))) != cudaSuccess) return e;
-    if ((e = cudaMemset(w, 0, sizeof(uint32_t))) != cudaSuccess) return e;
-    if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-    g_err_word[dev] = w;
+    // a variable of the module, zero when it is loaded: a first call may come from a stream that
+    // is being captured, where nothing can be allocated
+    void *w = nullptr;
+    RelaxedCapture relaxed;
+    if ((e = cudaGetSymbolAddress(&w, g_device_error)) != cudaSuccess) return e;
+    g_err_word[dev] = static_cast<uint32_t *>(w);
   }
   *word = g_err_word[dev];
   return cudaSuccess;
@@ -73,6 +82,7 @@ void keep_pool_memory(int dev) {
   static std::once_flag once[64];
   if (dev < 0 || dev >= 64) return;
   std::call_once(once[dev], [dev]() {
+    RelaxedCapture relaxed;
     cudaMemPool_t pool;
     if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
       uint64_t thr = ~0ull;

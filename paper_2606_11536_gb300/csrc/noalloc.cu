@@ -98,7 +98,7 @@ extern "C" pir_status_t pir_answer_noalloc(pir_db_t db, const uint32_t *queries,
   uint32_t *qhat = reinterpret_cast<uint32_t *>(b8 + out_bytes);
   void *qs = b8 + out_bytes + up256((size_t)B * Kc * 2 * L * n * 4);
 
-  // GEMM tile without the TMA scan (its error word is allocated on first use)
+  // the integer GEMM tiles: the scan and the digit GEMM take other query copies
   const uint32_t tile = limb ? 0 : (M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : 0);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint64_t launches = 0;
