@@ -274,6 +274,7 @@ cudaError_t fwd_any(const ParamCtx &c, const uint32_t *src, const RowMap &rm, co
 }  // namespace
 
 cudaError_t launch_ntt_fwd(const ParamCtx &c, const uint32_t *src, uint32_t *dst, uint64_t rows, cudaStream_t s) {
+  if (rows > kMaxRows) return cudaErrorInvalidValue;  // (a divisor past 2^31 has no FastDiv)
   const RawSrc rs = {};
   const RowMap rm(0, rows ? rows : 1, 0, 1, c.p.L);
   return fwd_any(c, src, rm, rs, dst, rows, s, false);

@@ -105,3 +105,15 @@ def test_captured_answers_between_other_kernels(gen, n, D1, D2, B, L):
             g.pir_graph_destroy(graph)
     finally:
         g.pir_free_db(db)
+
+
+def test_more_rows_than_there_can_be_are_refused():
+    """Counts past 2^31 rows of 8 KiB and more: an error from the host, with nothing launched."""
+    import ctypes as C
+
+    p = g.pir_make_params(2048, 8, 1, 1, 1)
+    x = torch.zeros(2048, dtype=torch.int32, device="cuda")
+    for count in (1 << 31, 1 << 40, (1 << 63) + 1, (1 << 64) - 1):
+        for f in (g.binding.lib().ntt_fwd, g.binding.lib().ntt_inv):
+            assert f(C.byref(p), C.c_void_p(x.data_ptr()), count, None) == 4
+    g.ntt_inv(p, g.ntt_fwd(p, x))
