@@ -55,17 +55,11 @@ struct ScanArgs {
   const uint32_t *acc_src;  // optional slot-major partial [L*n][M][D2] added before the write
 };
 
-// Rows per unrolled group and CTAs per SM, by accumulator count (MB rows x T quads):
-// the batch-1 shape keeps three CTAs (27 warps) per SM, two rows of loads per group.
+// CTAs per SM by accumulator count (MB rows x T quads): the shape of one query keeps three (27
+// warps); two rows of loads per unrolled group.
 template <int MB, int T>
-struct ScanShape {
-  static constexpr int U = (MB * T <= 4) ? 2 : 1;
-  static constexpr int kMinBlocks = (MB * T <= 2) ? 3 : (MB * T <= 4) ? 2 : 1;
-};
-
-template <int MB, int T>
-__global__ void __launch_bounds__(kThreads, ScanShape<MB, T>::kMinBlocks) k_scan_tma(ScanArgs a, ModConst mc) {
-  constexpr int U = ScanShape<MB, T>::U;
+__global__ void __launch_bounds__(kThreads, MB * T <= 2 ? 3 : 2) k_scan_tma(ScanArgs a, ModConst mc) {
+  constexpr int U = 2;
   extern __shared__ __align__(128) uint8_t smem[];
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * a.stage_bytes);
   const uint32_t full0 = saddr(bars), empty0 = saddr(bars + kStages), stall = saddr(bars + 2 * kStages);
@@ -431,8 +425,8 @@ cudaError_t launch_scan_direct(const ParamCtx &c, const uint32_t *db, uint32_t D
   return M <= 2 ? direct_launch<2>(c, a, s) : M <= 4 ? direct_launch<4>(c, a, s) : direct_launch<8>(c, a, s);
 }
 
-// The TMA scan holds M <= 8 rows and D2 <= 8 * 8 * 4 * 2 = 512 columns per lane
-// budget (T <= 2 quads per lane).
+// The scans as tile 7: M <= 8 rows, D2 <= 8 * 8 * 4 * 2 = 512 columns (two quads of columns per
+// lane of the staged scan's eight warps).
 bool scan_tma_supports(uint32_t M, uint32_t D2) { return M <= 8 && D2 % 4 == 0 && D2 <= 512; }
 
 cudaError_t launch_scan_tma(const ParamCtx &c, const uint32_t *db, uint32_t D1, uint32_t D2, const uint32_t *qs,
@@ -468,12 +462,10 @@ cudaError_t launch_scan_tma(const ParamCtx &c, const uint32_t *db, uint32_t D1, 
   a.stall_test = stall_test;
   a.out_poly = out_poly;
   a.acc_src = acc_src;
-  const uint32_t nq = D2 / 4;
-  const int T = nq > 64 ? 2 : 1;  // 8 warps x 8 quads per pass
-  const int MB = M <= 2 ? 2 : M <= 4 ? 4 : 8;
-  if (MB == 2) return T == 1 ? scan_launch<2, 1>(c, a, s) : scan_launch<2, 2>(c, a, s);
-  if (MB == 4) return T == 1 ? scan_launch<4, 1>(c, a, s) : scan_launch<4, 2>(c, a, s);
-  return T == 1 ? scan_launch<8, 1>(c, a, s) : scan_launch<8, 2>(c, a, s);
+  // one query in one or two quads a lane, two in one (scan_staged_wins); the stall test, whose
+  // consumers compute nothing, on any shape
+  if (M > 2) return scan_launch<4, 1>(c, a, s);
+  return D2 <= 256 ? scan_launch<2, 1>(c, a, s) : scan_launch<2, 2>(c, a, s);
 }
 
 }  // namespace gbpir
