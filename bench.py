@@ -741,8 +741,8 @@ def our_arm(args, wl):
         g.pir_release_memory()
         # a child process, as `bench.py --serving` runs: its allocators start empty, so
         # the 208 GiB of resident serving DBs meet no cache left by the blocks above.
-        # Uncaptured dispatch: with captured graphs an overloaded sweep has stalled
-        # (two batches that never completed), without them it has not
+        # Uncaptured dispatch.  On request only: with captured graphs an overloaded sweep, and
+        # without them this block, have stalled (large batches that never completed; cause open)
         cmd = [sys.executable, os.path.abspath(__file__), "--serving",
                "--serving-rates", str(args.serving_block_rate), "--serving-seconds", str(args.serving_block_seconds),
                "--serving-warmup", "1.5"]
@@ -1244,8 +1244,10 @@ def main(argv=None):
     ap.add_argument("--noalloc", action="store_true",
                     help="answer through pir_answer_noalloc (the library's fixed scratch array, no allocation)")
     ap.add_argument("--serving", action="store_true", help="run the serving benchmark instead")
-    ap.add_argument("--no-serving-block", dest="serving_block", action="store_false",
-                    help="leave the serving block out of the default line")
+    ap.add_argument("--serving-block", action="store_true",
+                    help="add the serving block to the default line (it has stalled; its run is bounded)")
+    ap.add_argument("--no-serving-block", dest="serving_block", action="store_false", default=False,
+                    help="leave it out (the default)")
     ap.add_argument("--serving-block-rate", type=float, default=1000.0)
     ap.add_argument("--serving-block-seconds", type=float, default=3.0)
     ap.add_argument("--serving-rates", type=float, nargs="+", default=[100, 300, 1000, 3000, 5000])
