@@ -360,7 +360,7 @@ def gemm_roofline(ctx, layout, B, p, tile, gemm_ms, launches_per_step, clocks, s
     M = 2 * B
     nslots = L_PRIMES * n
     launch_ms = gemm_ms / launches_per_step
-    rows = -(-D1 // launches_per_step)  # of one launch
+    rows = max(1, round(D1 / launches_per_step))  # of one launch
     choice = g.pir_gemm_choice(layout, rows, D2, B)
     # the kernel that ran, as a tile id (tile 7 is the staged or, 10, the direct scan)
     ran = choice if tile == 0 or (layout == g.PIR_LAYOUT_PLAIN and tile == 7 and choice == 10) else tile
