@@ -67,7 +67,7 @@ typedef enum {
   PIR_LAYOUT_PLAIN = 0,  /* u32 residues [L*n slots][D1][D2]: one query on the CUDA cores (u32 x u32 ->
                             u64), batches on the tensor cores (the words split into exact signed
                             base-256 f16 digits on the way, 1024-row f32 sums of at most 2^24);
-                            tiles 1-8 keep a batch on the CUDA cores */
+                            tiles 1-8 and 10 keep a batch on the CUDA cores */
   PIR_LAYOUT_LIMB = 1,   /* u8 limb planes [L*n slots][4][D2][D1]: the same tensor-core GEMM, the bytes
                             as f16 (512-row f32 sums below 2^24); tiles 1-3 run it on the INT8
                             tensor pipe (u8 x u8 -> s32)                                       */

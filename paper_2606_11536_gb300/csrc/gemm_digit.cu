@@ -675,7 +675,8 @@ cudaError_t launch_gemm_digit(const ParamCtx &c, int layout, const void *db, uin
   a.NH = H == 2 ? round16(NT / 2) : NT;
   a.R = H == 2 ? 3 : 2;
   const uint32_t CG = H == 2 || (NT >= 128 && D2 > 32) ? 2 : 1;
-  // column tiles per unit: as many as 128 accumulator columns hold, spread evenly
+  // column tiles per unit: as many as 128 accumulator columns hold, spread evenly.  The last unit
+  // runs its tiles past D2 too (132 columns: two units of three tiles, 192 columns of work)
   const uint32_t tiles = (D2 + 32 * CG - 1) / (32 * CG);
   const uint32_t tmax = a.NH > 64 ? 1 : 128 / a.NH;
   a.cgroups = (tiles + tmax - 1) / tmax;

@@ -40,7 +40,7 @@ __device__ __forceinline__ void byte_planes(uint32_t w0, uint32_t w1, uint32_t w
   p[3] = prmt(t1, t3, 0x7632);
 }
 
-// A tile: rows of KS bytes, 16-byte chunks XOR-swizzled by row (ldmatrix without
+// A tile: rows of KS bytes, 16-byte chunks XOR-swizzled by row (16-byte reads without
 // bank conflicts).
 __device__ __forceinline__ uint32_t swz_a(uint32_t r, uint32_t ch) { return r * KS + ((ch ^ (r & 7)) << 4); }
 // CUDA-core path: 256 rows per CTA (one per thread) x QB queries.  Per stage the raw

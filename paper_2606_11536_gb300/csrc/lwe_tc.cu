@@ -24,9 +24,9 @@
 //   8..23   converters, four warpgroups taking stages of 128 rows x 128 bytes in turn;
 //   24, 25  stream the DB and the query digits (tensor maps);
 //   26      issues the MMAs.
-// Measured (against mma.sync INT8, which this replaced): 1 GiB DB (32768 x 32768), 32 queries
-// 2265 -> 197 us, 5.5 TB/s of DB; 8 GiB DB, 16 queries 1273 us, 6.7 TB/s = the measured copy
-// rate.  Bound by HBM up to 16 queries; at 32 an MMA (74 cycles per 2 KiB of DB) is close
+// Measured (whole calls, against mma.sync INT8, which this replaced): 1 GiB DB (32768 x 32768), 32
+// queries 2265 -> 215 us, 5.0 TB/s of DB; 8 GiB DB, 16 queries 1273 us, 6.7 TB/s = the measured
+// copy rate.  Bound by HBM up to 16 queries; at 32 an MMA (74 cycles per 2 KiB of DB) is close
 // behind the stream (87).
 // Every barrier wait is bounded; one that runs out sets the device error word.
 #include "async.cuh"

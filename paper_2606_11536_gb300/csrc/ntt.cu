@@ -19,10 +19,11 @@
 // Output order: forward NTT(a)[k] = sum_t a_t psi^((2 brv(k) + 1) t), the natural
 // result of decimation in time with psi powers in bit-reversed order.
 //
-// Bound by the multiply-add pipe (a butterfly's high product and two low ones) and the
-// issue slots around it: 2 GiB of rows, n = 2^12, forward 1393 -> 1140 us (3.8 TB/s), n = 2^13,
-// inverse 1610 -> 1315 us, with row numbers divided by multiplication instead of 64-bit
-// divisions (a sixth of all instructions), one block barrier a row, whole-sector stores.
+// Bound by the multiply-add pipe (a butterfly's high product and two low ones; 71 to 73% active),
+// the shared-memory wavefronts (64 to 70%) and the issue slots (66%) together: 2 GiB of rows,
+// n = 2^12, forward 1393 -> 1140 us (3.8 TB/s), n = 2^13, inverse 1610 -> 1315 us, with row numbers
+// divided by multiplication instead of 64-bit divisions (a sixth of all instructions), one block
+// barrier a row, whole-sector stores.
 #include "ntt_row.cuh"
 
 namespace gbpir {

@@ -12,7 +12,8 @@
 // output of each butterfly that leads to its slots (n = 2^12: 40 butterfly outputs' products
 // where one CTA would take 32).  The CTAs of a row are neighbours and share its read in L2.
 //
-// Bound by issue slots (56%) and shared-memory wavefronts (67%), the transform's and the digits'.
+// No unit is full (n = 2^11: shared-memory wavefronts 65%, issue 47%, multiply-add pipe 46%, DRAM
+// 44%): phases of loads, transform, digits and stores between block barriers.
 // Transform and transpose -> this: n = 2^12, 32 queries x 2048 x L = 2 4.80 -> 4.04 ms (12.9 GB), bf16
 // 32 x 512 1201 -> 993 us; n = 2^11, 32 x 512 605 -> 489 us; L = 3, 3 x 301 134 -> 101 us.  Three CTAs per SM
 // at 40 registers for n >= 2^12; n = 2^11 spills there and takes two (620 -> 489 us).
