@@ -1,6 +1,6 @@
 """Compile the C oracle into ``oracle/libpir_oracle.so`` (gcc, no GPU, any arch).
 
-Test infrastructure: building the checker is not using it.
+Test infrastructure: building the oracle is not using it.
 """
 from __future__ import annotations
 
